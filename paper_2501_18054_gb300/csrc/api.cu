@@ -77,7 +77,7 @@ Layout make_layout(const pngf_config& cfg) {
   L.gsplit = take(mixed ? n * n * 4 * sizeof(float) : 0);
   L.xs = take(mixed ? (1 + n_o) * n * 8 * sizeof(float) : 0);
   L.xadd = take(mixed ? (size_t)L.R * 4 * sizeof(float) : 0);  // alpha_i of the mixed search as double-words
-  L.ipiv = take(2 * n * sizeof(int));
+  L.oz = take(pec ? 0 : factor_scratch_bytes(cfg.n_d));
   L.snapW = take(L.snapW_bytes);
   L.snapState = take(L.state_bytes + sizeof(Control));
   L.ctl = take(sizeof(Control));
@@ -179,7 +179,6 @@ pngf_status pngf_factor(pngf_ctx* c, const uint8_t* b) {
     return st;
   }
   pngf_status st = factor_fp64(c, b);
-  if (st == PNGF_OK && c->cfg.precision == PNGF_MIXED) st = mixed_after_factor(c);
   if (st == PNGF_OK) c->factored = true;
   return st;
 }

@@ -703,17 +703,6 @@ __global__ void __launch_bounds__(kThreads) dbs_mixed_kernel(SweepArgs a) {
   }
 }
 
-// ---------------------------------------------------------------- after the factor
-__global__ void to_planar_fp32(const c128* __restrict__ W, int n, int ldw, float* __restrict__ Wr,
-                               float* __restrict__ Wi, int ldl) {
-  int i = blockIdx.y;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    c128 w = W[(size_t)i * ldw + j];
-    Wr[(size_t)i * ldl + j] = (float)w.x;
-    Wi[(size_t)i * ldl + j] = (float)w.y;
-  }
-}
-
 // ---------------------------------------------------------------- single calls
 __global__ void mixed_accept_kernel(SweepArgs a, int k) {
   __shared__ Pivot s_pv;
@@ -774,15 +763,6 @@ __global__ void flush_reset_kernel(SweepArgs a) {
 
 
 }  // namespace
-
-pngf_status mixed_after_factor(pngf_ctx* c) {
-  const int n = c->cfg.n_d;
-  dim3 grid((n + 255) / 256 > 8 ? 8 : (n + 255) / 256, n);
-  to_planar_fp32<<<grid, 256, 0, c->stream>>>(at<c128>(c, c->L.W), n, c->L.ldw, at<float>(c, c->L.Wlo_re),
-                                                at<float>(c, c->L.Wlo_im), c->L.ldl);
-  return cuda_status(cudaGetLastError());
-}
-
 
 static void* mixed_kernel_for(int objective) {
   return objective == PNGF_OBJ_MAX_WEIGHTED_POWER ? (void*)dbs_mixed_kernel<PNGF_OBJ_MAX_WEIGHTED_POWER>
