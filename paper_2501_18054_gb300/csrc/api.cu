@@ -6,7 +6,7 @@
 #include <cstring>
 #include <new>
 
-#include "flush_tc.cuh"
+#include "delayed64.cuh"
 
 namespace pngf {
 
@@ -77,7 +77,18 @@ Layout make_layout(const pngf_config& cfg) {
   L.gsplit = take(mixed ? n * n * 4 * sizeof(float) : 0);
   L.xs = take(mixed ? (1 + n_o) * n * 8 * sizeof(float) : 0);
   L.xadd = take(mixed ? (size_t)L.R * 4 * sizeof(float) : 0);  // alpha_i of the mixed search as double-words
-  L.oz = take(pec ? 0 : factor_scratch_bytes(cfg.n_d));
+  const bool fp64 = cfg.precision == PNGF_FP64;
+  L.oz = take(fp64 ? factor_scratch_bytes(cfg.n_d) : mixed ? 2 * n * sizeof(int) : 0);  // mixed: the pivots
+  if (fp64) {
+    size_t im[4];
+    factor_images(cfg.n_d, im);
+    L.ozA = L.oz + im[0];
+    L.ozB = L.oz + im[1];
+    L.ozEa = L.oz + im[2];
+    L.ozEb = L.oz + im[3];
+  }
+  L.X64 = take(fp64 ? (size_t)kDelay64 * L.ldt * c : 0);
+  L.last64 = take(fp64 ? n * sizeof(int) : 0);
   L.snapW = take(L.snapW_bytes);
   L.snapState = take(L.state_bytes + sizeof(Control));
   L.ctl = take(sizeof(Control));
@@ -178,7 +189,7 @@ pngf_status pngf_factor(pngf_ctx* c, const uint8_t* b) {
     if (st == PNGF_OK) c->factored = true;
     return st;
   }
-  pngf_status st = factor_fp64(c, b);
+  pngf_status st = c->cfg.precision == PNGF_MIXED ? factor_mixed(c, b) : factor_fp64(c, b);
   if (st == PNGF_OK) c->factored = true;
   return st;
 }

@@ -27,6 +27,7 @@
 // digits 2.5.
 #include <cstdio>
 
+#include "form_ports.cuh"
 #include "ozaki.cuh"
 
 namespace pngf {
@@ -38,7 +39,7 @@ constexpr int FT_THREADS = OZ_THREADS;
 constexpr int FT_WARPS = FT_THREADS / 32;
 
 struct FactorArgs {
-  int n, n_o, ldw, ldt, ldl;
+  int n, n_o, ldw, ldt;
   const c128* G;
   const c128* God;
   const c128* cd;
@@ -52,9 +53,6 @@ struct FactorArgs {
   c128* diag;
   c128* e;
   double* Gs;  // Re G + Im G
-  float4* G2;  // mixed: G as FP32 pairs
-  float* Wr;   // mixed: planar FP32 copy of W
-  float* Wi;
   int* act;    // the m pixels that are on, ascending, then the n - m others
   int* count;  // m
   unsigned char* imgA;
@@ -349,8 +347,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
   OzState oz;
   oz_setup(oz, s_bars, &s_tmem);
   bool ok = true;
-  // ---- the lists (CTA 0); one pass over G: Re G + Im G and the FP32 pairs of
-  //      the refreshes; the rows of W at pixels that are off start as [G | c_d]
+  // ---- the lists (CTA 0); one pass over G: Re G + Im G for the refreshes; the rows of W at pixels that are off start as [G | c_d]
   if (cta == 0) factor_lists(a);
   for (int i = cta; i < n; i += P) {
     const c128* g = a.G + (size_t)i * n;
@@ -361,10 +358,6 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
       const c128 z = g[j];
       if (!on) w[j] = z;
       gs[j] = z.x + z.y;
-      if (a.G2) {  // hi = fl32(g), lo = fl32(g - hi)
-        const float rh = (float)z.x, ih = (float)z.y;
-        a.G2[(size_t)i * n + j] = make_float4(rh, ih, (float)(z.x - (double)rh), (float)(z.y - (double)ih));
-      }
     }
     if (tid == 0) {
       if (!on) w[n] = a.cd[i];
@@ -577,8 +570,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
       if (ok) ok = grid_sync(ctl);
     }
   }
-  // ---- the lower triangle of W mirrors the upper one; diag W, e and the mixed
-  //      path's planes are read off on the way
+  // ---- the lower triangle of W mirrors the upper one; diag W and e are read off
   if (ok) {
     constexpr int TS = 32, TLD = TS + 1;
     const int nt = (n + TS - 1) / TS;
@@ -593,22 +585,13 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
           const c128 w = a.W[(size_t)i * ldw + j];
           sm[r * TLD + c] = w;
           if (i == j) a.diag[i] = w;
-          if (a.Wr && i <= j) {
-            a.Wr[(size_t)i * a.ldl + j] = (float)w.x;
-            a.Wi[(size_t)i * a.ldl + j] = (float)w.y;
-          }
         }
       }
       __syncthreads();
       for (int q = tid; q < TS * TS; q += FT_THREADS) {
         const int r = q / TS, c = q % TS, i = bj * TS + r, j = bi * TS + c;  // lower: i > j
         if (i < n && j < i) {
-          const c128 w = sm[c * TLD + r];
-          a.W[(size_t)i * ldw + j] = w;
-          if (a.Wr) {
-            a.Wr[(size_t)i * a.ldl + j] = (float)w.x;
-            a.Wi[(size_t)i * a.ldl + j] = (float)w.y;
-          }
+          a.W[(size_t)i * ldw + j] = sm[c * TLD + r];
         }
       }
     }
@@ -617,38 +600,6 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
     latch_status(ctl, PNGF_ETIMEOUT);
   }
   oz_teardown(oz, !ok);
-}
-
-// o = c_o + G_od (v .* e), objective, reset of the sweep counters.  One CTA.
-__global__ void __launch_bounds__(256) form_o(const c128* __restrict__ God, const c128* __restrict__ co,
-                                              const c128* __restrict__ v, const c128* __restrict__ e,
-                                              int n, ObjParams op, Control* __restrict__ ctl) {
-  __shared__ c128 red[kMaxPorts][256];
-  c128 acc[kMaxPorts];
-  for (int p = 0; p < kMaxPorts; ++p) acc[p] = mk(0.0, 0.0);
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    c128 ve = cmul(v[j], e[j]);
-    FOR_PORTS(p, op.n_o) acc[p] = cfma(God[(size_t)p * n + j], ve, acc[p]);
-  }
-  FOR_PORTS(p, op.n_o) red[p][threadIdx.x] = acc[p];
-  __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if (threadIdx.x < s)
-      FOR_PORTS(p, op.n_o) red[p][threadIdx.x] = cadd(red[p][threadIdx.x], red[p][threadIdx.x + s]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    c128 o[kMaxPorts];
-    FOR_PORTS(p, op.n_o) {
-      o[p] = cadd(co[p], red[p][0]);
-      ctl->o[p] = o[p];
-    }
-    ctl->f = objective_of(op, o);
-    ctl->factored = 1;
-    ctl->n_acc_total = 0;
-    ctl->since_refresh = 0;
-    ctl->r_delay = 0;
-  }
 }
 
 }  // namespace
@@ -683,6 +634,13 @@ static FactorScratch factor_scratch(int n) {
   return f;
 }
 size_t factor_scratch_bytes(int n) { return factor_scratch(n).total; }
+void factor_images(int n, size_t off[4]) {
+  const FactorScratch f = factor_scratch(n);
+  off[0] = f.imgA;
+  off[1] = f.imgB;
+  off[2] = f.ea;
+  off[3] = f.eb;
+}
 
 // ---------------------------------------------------------------- driver
 pngf_status factor_fp64(pngf_ctx* c, const uint8_t* b) {
@@ -690,13 +648,11 @@ pngf_status factor_fp64(pngf_ctx* c, const uint8_t* b) {
   cudaStream_t s = c->stream;
   const FactorScratch f = factor_scratch(n);
   char* ws = c->ws + c->L.oz;
-  const bool mixed = c->cfg.precision == PNGF_MIXED;
   FactorArgs a{};
   a.n = n;
   a.n_o = c->cfg.n_o;
   a.ldw = c->L.ldw;
   a.ldt = c->L.ldt;
-  a.ldl = c->L.ldl;
   a.G = c->G;
   a.God = c->God;
   a.cd = c->cd;
@@ -710,9 +666,6 @@ pngf_status factor_fp64(pngf_ctx* c, const uint8_t* b) {
   a.diag = at<c128>(c, c->L.diag);
   a.e = at<c128>(c, c->L.e);
   a.Gs = at<double>(c, c->L.gsum);
-  a.G2 = mixed ? at<float4>(c, c->L.gsplit) : nullptr;
-  a.Wr = mixed ? at<float>(c, c->L.Wlo_re) : nullptr;
-  a.Wi = mixed ? at<float>(c, c->L.Wlo_im) : nullptr;
   a.imgA = reinterpret_cast<unsigned char*>(ws + f.imgA);
   a.imgB = reinterpret_cast<unsigned char*>(ws + f.imgB);
   a.ea = reinterpret_cast<int*>(ws + f.ea);

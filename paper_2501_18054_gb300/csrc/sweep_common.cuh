@@ -9,6 +9,7 @@ namespace pngf {
 namespace {
 
 constexpr int kThreads = 512;
+constexpr int kMaxWarps = 18;  // of any CTA that uses the helpers below (their per-warp arrays)
 // Bound of every device-side wait on other CTAs: at most 2^24 polls (or a
 // context's own count, Control::spin_limit, set by pngf_set_wait_limit) and
 // at most kWaitNs of wall-clock time on the GPU's global timer, whichever
@@ -71,6 +72,13 @@ struct SweepArgs {
   int* actg;                  // n: active-pixel list of the last refresh (written by CTA 0)
   const float4* G2;           // n x n: G as FP32 pairs (Re hi, Im hi, Re lo, Im lo)
   float4* xs;                 // (1 + n_o) x n x 2: x = v.[e, T] at the active pixels, FP32 pairs, each part twice
+  // FP64 path: the delayed set (column i at X64 + i ldt) and the fold's operand images
+  c128* X64;
+  int* last64;  // n: index of the pixel's last flip in the set, -1: none
+  unsigned char* ozA;
+  unsigned char* ozB;
+  int* ozEa;
+  int* ozEb;
   float4* xadd;               // R: alpha_i of the mixed search as double-word pairs, until copied to xa
 };
 
@@ -162,7 +170,7 @@ __device__ __forceinline__ unsigned long long sel_read(Control* ctl, int rd) {
 
 // ---------------------------------------------------------------- block reductions
 __device__ long long block_min_ll(long long x) {
-  __shared__ long long sh[kThreads / 32];
+  __shared__ long long sh[kMaxWarps];
   for (int off = 16; off > 0; off >>= 1) x = min(x, __shfl_down_sync(0xffffffffu, x, off));
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   __syncthreads();
@@ -183,8 +191,8 @@ __device__ __forceinline__ bool better(double g1, int p1, double g2, int p2) {
 }
 
 __device__ void block_best(double& g, int& p) {
-  __shared__ double shg[kThreads / 32];
-  __shared__ int shp[kThreads / 32];
+  __shared__ double shg[kMaxWarps];
+  __shared__ int shp[kMaxWarps];
   for (int off = 16; off > 0; off >>= 1) {
     double og = __shfl_down_sync(0xffffffffu, g, off);
     int op = __shfl_down_sync(0xffffffffu, p, off);
@@ -400,7 +408,7 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 // Ascending list of the pixels with b_i = 1 (the only nonzero entries of
 // x = v.[e, T]) in shared memory act[0, m); returns m (the same in every thread).
 __device__ int active_list(const SweepArgs& a, int* act) {
-  __shared__ int s_scan[kThreads / 32];
+  __shared__ int s_scan[kMaxWarps];
   __shared__ int s_m;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int chunk = (a.n + blockDim.x - 1) / blockDim.x;
@@ -603,7 +611,7 @@ __device__ __forceinline__ void correct_upper(const SweepArgs& a, int pb, int pe
 // with the active list act[0, m) only those rows of the strip are read.
 template <int NV, bool MIXED>
 __device__ __noinline__ void refresh_correct_t(const SweepArgs& a, int pb, int pe, const int* act, int m) {
-  __shared__ f2c red[kThreads / 32][32];
+  __shared__ f2c red[kMaxWarps][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   correct_upper<NV, MIXED>(a, pb, pe);
   __syncthreads();
@@ -882,7 +890,7 @@ __device__ void correct_strips(const SweepArgs& a, int pb, int pe, const int* ac
 
 // partial o sums of pixels [pb, pe) -> opart[cta]
 __device__ __noinline__ void ports_partial(const SweepArgs& a, int pb, int pe) {
-  __shared__ c128 red[kMaxPorts][kThreads / 32];
+  __shared__ c128 red[kMaxPorts][kMaxWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int p = 0; p < a.n_o; ++p) {
     c128 acc = mk(0.0, 0.0);
@@ -962,6 +970,12 @@ SweepArgs make_args(pngf_ctx* c) {
   a.G2 = a.mixed ? at<float4>(c, L.gsplit) : nullptr;
   a.xs = a.mixed ? at<float4>(c, L.xs) : nullptr;
   a.xadd = a.mixed ? at<float4>(c, L.xadd) : nullptr;
+  a.X64 = at<c128>(c, L.X64);
+  a.last64 = at<int>(c, L.last64);
+  a.ozA = reinterpret_cast<unsigned char*>(c->ws + L.ozA);
+  a.ozB = reinterpret_cast<unsigned char*>(c->ws + L.ozB);
+  a.ozEa = at<int>(c, L.ozEa);
+  a.ozEb = at<int>(c, L.ozEb);
   a.tensor_fold = c->cfg.precision == PNGF_MIXED && c->cfg.tensor_fold;
   a.tcimgA = reinterpret_cast<unsigned char*>(c->ws) + L.tcimg;
   a.tcimgB = a.tcimgA + L.tcimgA_bytes;
