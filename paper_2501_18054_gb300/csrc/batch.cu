@@ -23,7 +23,7 @@
 #include <algorithm>
 #include <vector>
 
-#include "flush_tc.cuh"
+#include "delayed64.cuh"
 #include "rank1.cuh"
 
 namespace pngf {
@@ -33,7 +33,7 @@ constexpr int kBatchThreads = 256;
 
 // o = c_o + G_od (v .* e) over all pixels of the run (CTA-local reduction)
 __device__ void cta_ports(const SweepArgs& a, const ObjParams& op, c128* s_o, double* s_f) {
-  __shared__ c128 red[kBatchThreads / 32];
+  __shared__ c128 red[kMaxWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int p = 0; p < a.n_o; ++p) {
     c128 acc = mk(0.0, 0.0);
@@ -305,6 +305,231 @@ __global__ void __launch_bounds__(kBatchThreads, 2) dbs_batch_kernel(const Sweep
   if (use_tc) tc_teardown(tcs, tc_failed);
 }
 
+// ---------------------------------------------------------------- FP64, FIRST mode
+// The delayed search of delayed64.cuh with one CTA per run: only CTA-wide
+// barriers, the folds on this SM's tensor core.  The visiting positions are
+// scored kScoreChunk at a time from the current one (a scoring warp on each SM
+// sub-partition; a flip is kept every few positions early in a search).
+// Bound by the SM's FP64 pipe (the columns: r complex multiply-adds per pixel)
+// and the read-back of the folds.  96 lossy-metal runs of 256, 576 and 1024
+// pixels, three sweeps: 734 -> 112 ms (before: the triangle's rank-1 update on
+// the FP64 pipe, 0.6 ms per kept flip of a 1024-pixel run).
+constexpr int kScoreChunk = 128;
+
+// the refresh of a whole run by one CTA; smem: the active-pixel list, then the
+// staging of the correction (OZ_SMEM bytes)
+__device__ void cta_refresh64(const SweepArgs& a, const ObjParams& op, c128* s_o, double* s_f, unsigned char* smem) {
+  int* act = reinterpret_cast<int*>(smem);
+  __syncthreads();
+  refresh_x(a, 0, a.n);
+  __syncthreads();
+  const int m = refresh_residual(a, 0, a.n, act);
+  for (int t = threadIdx.x; t < m; t += blockDim.x) a.actg[t] = act[t];
+  const int t_end = count_below(act, m, a.n - 1);
+  __syncthreads();
+  correct_strips<false>(a, 0, a.n, a.actg, t_end, reinterpret_cast<float*>(smem), OZ_SMEM);
+  __syncthreads();
+  cta_ports(a, op, s_o, s_f);
+}
+
+__global__ void __launch_bounds__(OZ_THREADS, 1) dbs_batch_fp64_kernel(const SweepArgs* __restrict__ runs, int n_runs,
+                                                                       int* __restrict__ queue) {
+  extern __shared__ __align__(128) unsigned char b_smem[];
+  constexpr int NW = OZ_THREADS / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ c128 s_o[kMaxPorts], s_alpha, s_coef, s_Tk[kMaxPorts];
+  __shared__ double s_f;
+  __shared__ ObjParams s_op;
+  __shared__ c128 s_beta[kDelay64], s_al[kDelay64], s_invd[kDelay64];
+  __shared__ int s_hist[kDelay64];
+  __shared__ int s_best, s_k, s_bad, s_run;
+  __shared__ __align__(8) unsigned long long s_bars[OZ_NBAR];
+  __shared__ unsigned s_tmem;
+  OzState oz;
+  oz_setup(oz, s_bars, &s_tmem);
+  bool oz_failed = false;
+  while (!oz_failed) {
+    __syncthreads();  // every thread has read the previous s_run
+    if (tid == 0) s_run = atomicAdd(queue, 1);
+    __syncthreads();
+    const int run = s_run;
+    if (run >= n_runs) break;
+    const SweepArgs& a = runs[run];
+    const int n = a.n, n_o = a.n_o;
+    const size_t ldx = a.ldt;
+    Control* ctl = a.ctl;
+    if (tid == 0) {
+      s_op = a.op;
+      FOR_PORTS(p, n_o) s_o[p] = ctl->o[p];
+      s_f = ctl->f;
+      s_best = INT_MAX;
+      s_bad = 0;
+    }
+    for (int q = tid; q < n; q += blockDim.x) a.last64[q] = -1;
+    __syncthreads();
+    long long n_acc = 0, n_evals = 0, n_refresh = 0;
+    int sweeps_done = 0, converged = 0, status = PNGF_OK;
+    int since_refresh = ctl->since_refresh;
+    int s = 0, t = 0, acc_in_sweep = 0, r = 0;
+    auto fold = [&]() -> bool {
+      if (r == 0) return true;
+      __syncthreads();
+      fold64_digits(a.X64, ldx, s_al, a.last64, r, n, a.ozA, a.ozB, a.ozEa, a.ozEb, warp, NW);
+      fold64_bases(a.W, a.ldw, a.X64, ldx, s_invd, s_hist, a.last64, r, n, tid, blockDim.x);
+      __syncthreads();
+      const bool ok = fold64_product(oz, b_smem, a.W, a.ldw, n, r, a.ozA, a.ozB, a.ozEa, a.ozEb, 0, 1);
+      for (int q = tid; q < n; q += blockDim.x) {
+        a.last64[q] = -1;
+        a.diag[q] = a.W[(size_t)q * a.ldw + q];  // d is formed from the matrix's own diagonal
+      }
+      __syncthreads();
+      r = 0;
+      return ok;
+    };
+    while (true) {
+      // ---- score a chunk of positions
+      const int chunk_end = min(n, t + kScoreChunk);
+      double fn = 0.0;
+      c128 al = mk(0.0, 0.0), co = al, idv = al;
+      int pos = INT_MAX, j = 0;
+      if (tid < kScoreChunk) {
+        const int q = t + tid;
+        if (q < n) {
+          const double f = s_f, thr = accept_threshold(s_op, f);
+          j = a.order ? a.order[(size_t)s * n + q] : q;
+          if ((unsigned)j >= (unsigned)n) s_bad = 1;
+          else if (score_flip64(s_op, a.dv[j], a.b[j] != 0, a.diag[j], a.e[j],
+                                [&](int p) { return a.T[(size_t)p * a.ldt + j]; }, s_o, fn, al, co, idv) &&
+                   improves64(s_op, fn, f, thr))
+            pos = q;
+        }
+        const int wmin = __reduce_min_sync(0xffffffffu, pos);
+        if (lane == 0 && wmin != INT_MAX) atomicMin(&s_best, wmin);
+      }
+      __syncthreads();
+      const int best = s_best;
+      if (s_bad) {
+        status = PNGF_EINVAL;
+        break;
+      }
+      if (best == INT_MAX) {
+        n_evals += chunk_end - t;
+        t = chunk_end;
+        if (t < n) continue;
+        ++sweeps_done;
+        if (acc_in_sweep == 0) { converged = 1; break; }
+        ++s;
+        if (s >= a.n_sweeps) break;
+        if (!fold()) { oz_failed = true; break; }
+        t = 0;
+        acc_in_sweep = 0;
+        continue;
+      }
+      // ---- the kept flip; o and f exactly as the scorer formed them
+      if (pos == best) {
+        s_k = j;
+        s_alpha = al;
+        s_coef = co;
+        s_al[r] = al;
+        s_invd[r] = idv;
+        s_hist[r] = j;
+        s_f = fn;
+        for (int p = 0; p < n_o; ++p) {
+          const c128 tk = a.T[(size_t)p * a.ldt + j];
+          s_Tk[p] = tk;
+          s_o[p] = cfma(co, tk, s_o[p]);
+        }
+        if (n_acc < a.trace_cap) {
+          if (a.trace) {
+            int32_t* tr = a.trace + 4 * n_acc;
+            tr[0] = s;
+            tr[1] = best;
+            tr[2] = j;
+            tr[3] = 0;
+          }
+          if (a.trace_f) a.trace_f[n_acc] = fn;
+        }
+      }
+      if (n_acc >= a.trace_cap && status == PNGF_OK) status = PNGF_ECAPACITY;
+      n_evals += best - t + 1;
+      t = best + 1;
+      ++n_acc;
+      ++acc_in_sweep;
+      __syncthreads();
+      const int k = s_k;
+      if (tid == 0) s_best = INT_MAX;
+      if (oz_exp(s_f) == 0x7ff) status = PNGF_ENUMERIC;
+      const int lk = a.last64[k];
+      for (int i = tid; i < r; i += blockDim.x)
+        s_beta[i] = i > lk ? cmul(s_al[i], a.X64[(size_t)i * ldx + k]) : mk(0.0, 0.0);
+      __syncthreads();
+      // ---- the column and the state of every pixel (a warp per 32 pixels, so
+      //      that an entry's chains, its column entry and its state stay on one lane)
+      const c128 alpha = s_alpha, coef = s_coef;
+      for (int q = tid; q < n; q += blockDim.x) {
+        const int lj = a.last64[q];
+        const c128 w = q == k ? a.diag[q] : delayed_base(a.W, a.ldw, k, q, lk, lj, s_invd, [&](int i, int p) {
+          return a.X64[(size_t)i * ldx + p];
+        });
+        c128 ch[kChains64];
+#pragma unroll
+        for (int p = 0; p < kChains64; ++p) ch[p] = delayed_chain(s_beta, a.X64 + q, ldx, p, q == k ? r : lj, r);
+        const c128 c = delayed_entry(w, ch, 1), ac = cmul(alpha, c), idk = s_invd[r];
+        a.X64[(size_t)r * ldx + q] = c;
+        // pixel k itself: y + alpha W_kk y = y / d
+        a.diag[q] = q == k ? cmul(a.diag[q], idk) : cfma(ac, c, a.diag[q]);
+        a.e[q] = q == k ? cmul(a.e[q], idk) : cfma(coef, c, a.e[q]);
+#pragma unroll 1
+        for (int p = 0; p < n_o; ++p) {
+          c128* tp = a.T + (size_t)p * a.ldt + q;
+          *tp = q == k ? cmul(*tp, idk) : cfma(ac, s_Tk[p], *tp);
+        }
+        if (q == k) {
+          const uint8_t nb = a.b[q] ^ 1;
+          a.b[q] = nb;
+          a.v[q] = nb ? a.dv[q] : mk(0.0, 0.0);
+          a.last64[q] = r;
+        }
+      }
+      __syncthreads();
+      ++r;
+      ++since_refresh;
+      const bool refresh = a.refresh_k > 0 && since_refresh >= a.refresh_k;
+      if (r == kDelay64 || refresh || t >= n) {
+        if (!fold()) { oz_failed = true; break; }
+      }
+      if (refresh) {
+        since_refresh = 0;
+        ++n_refresh;
+        cta_refresh64(a, s_op, s_o, &s_f, b_smem);
+      }
+      if (status == PNGF_ENUMERIC) break;
+      if (t >= n) {
+        ++sweeps_done;
+        ++s;
+        if (s >= a.n_sweeps) break;
+        t = 0;
+        acc_in_sweep = 0;
+      }
+    }
+    if (!oz_failed && !fold()) oz_failed = true;  // what a break left in the set
+    if (oz_failed) status = PNGF_ETIMEOUT;
+    __syncthreads();
+    if (tid == 0) {
+      FOR_PORTS(p, n_o) ctl->o[p] = s_o[p];
+      ctl->f = s_f;
+      ctl->since_refresh = since_refresh;
+      ctl->n_acc_total += (int)n_acc;
+      const long long cnt[8] = {n_acc, n_evals, sweeps_done, converged, n_refresh, 0, status, 0};
+      for (int q = 0; q < 8; ++q) ctl->counters[q] = cnt[q];
+      if (a.counters)
+        for (int q = 0; q < 8; ++q) a.counters[q] = cnt[q];
+      if (status == PNGF_ENUMERIC || status == PNGF_EINVAL || status == PNGF_ETIMEOUT) latch_status(ctl, status);
+    }
+  }
+  oz_teardown(oz, oz_failed);
+}
+
 // The per-run argument table is written by the device from kernel parameters
 // (chunks of the table passed by value), so that no host buffer has to outlive
 // the call: a stream capture records the values themselves.
@@ -356,13 +581,19 @@ pngf_status run_sweep_batch(pngf_ctx* const* ctxs, int n_runs, int n_sweeps, con
     if (cudaGetLastError() != cudaSuccess) return PNGF_ECUDA;
   }
   const bool mixed = c0->cfg.precision == PNGF_MIXED;
+  if (cudaMemsetAsync(queue, 0, sizeof(int), c0->stream) != cudaSuccess) return PNGF_ECUDA;
+  int grid = c0->n_sm;  // one CTA per SM
+  if (grid > n_runs) grid = n_runs;
+  if (!mixed && c0->cfg.mode == PNGF_FIRST_IMPROVEMENT) {
+    if (cudaFuncSetAttribute(dbs_batch_fp64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM) != cudaSuccess)
+      return PNGF_ECUDA;
+    dbs_batch_fp64_kernel<<<grid, OZ_THREADS, OZ_SMEM, c0->stream>>>(static_cast<const SweepArgs*>(ws), n_runs, queue);
+    return cuda_status(cudaGetLastError());
+  }
   size_t smem = mixed ? (kFlushSmem > (size_t)tc_fold_smem(1) ? kFlushSmem : (size_t)tc_fold_smem(1))
                       : 2 * (size_t)max_n * sizeof(c128);
   if (cudaFuncSetAttribute(dbs_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return PNGF_ECUDA;
-  if (cudaMemsetAsync(queue, 0, sizeof(int), c0->stream) != cudaSuccess) return PNGF_ECUDA;
-  int grid = c0->n_sm;  // one CTA per SM
-  if (grid > n_runs) grid = n_runs;
   dbs_batch_kernel<<<grid, kBatchThreads, smem, c0->stream>>>(static_cast<const SweepArgs*>(ws), n_runs, queue);
   return cuda_status(cudaGetLastError());
 }
