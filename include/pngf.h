@@ -80,9 +80,10 @@ typedef enum {
  * stay within about 1e+-38), refreshed against G every refresh_k flips.
  * PNGF_PEC: FP64, pixels of perfect electric conductor (the paper's binary
  * system, Eq. 2, [(I - P) + P G] j = P e_inc; dv is not used): the search
- * keeps H = (G_MM)^-1 of the metal set M, Q = G H and W = G - G H G, and a
- * flip is a symmetric rank-1 change of H and W and a rank-1 change of Q; the
- * state of a design is built from the empty design by rank-1 additions
+ * keeps the parts of H = (G_MM)^-1 (metal set M), Q = G H and W = G - G H G
+ * that are not zero in one complex symmetric matrix, of which a flip is a
+ * rank-1 change; the state of a design is built from the empty design by
+ * rank-1 additions
  * (pngf_factor).  No refresh (refresh_k is ignored); pngf_set_state,
  * pngf_gradient, pngf_score_flips' o_new, the batch and tile calls are not
  * available (PNGF_EINVAL).  pngf_get_state returns W (upper triangle current),

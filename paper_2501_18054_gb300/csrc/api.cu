@@ -30,15 +30,14 @@ Layout make_layout(const pngf_config& cfg) {
   };
   const size_t c = sizeof(c128);
   L.W = take(n * L.ldw * c);
-  L.LU = take(n * L.ldw * c);  // PEC: H = (G_MM)^-1 padded
-  L.Q = take(pec ? n * L.ldw * c : 0);  // PEC: Q = G H (full)
+  L.LU = take(pec ? 0 : n * L.ldw * c);
   // mixed path: [Wlo_re | Wlo_im | X | xa] contiguous, so one copy snapshots them
   const size_t plane = n * L.ldl * sizeof(float);
   L.Wlo_re = take(mixed ? 2 * plane : 0);
   L.Wlo_im = L.Wlo_re + (mixed ? plane : 0);
   L.X = take(n * (size_t)L.R * 2 * sizeof(float));
   L.xa = take((size_t)L.R * c);
-  L.snapW_bytes = mixed ? off - L.Wlo_re : pec ? off - L.W : n * L.ldw * c;  // PEC: W, H, Q contiguous
+  L.snapW_bytes = mixed ? off - L.Wlo_re : n * L.ldw * c;
   // contiguous state block: diag, e, T, v, b
   L.diag = off;
   off += align_up(n * c, 256);
@@ -50,14 +49,6 @@ Layout make_layout(const pngf_config& cfg) {
   off += align_up(n * c, 256);
   L.b = off;
   off += align_up(n, 256);
-  if (pec) {  // PEC: current j, R = G_od H, diag H
-    L.pj = off;
-    off += align_up(n * c, 256);
-    L.pR = off;
-    off += align_up(n_o * L.ldt * c, 256);
-    L.pdiagH = off;
-    off += align_up(n * c, 256);
-  }
   L.state_bytes = off - L.diag;
   L.pos_of = take(n * sizeof(int));
   L.part = take((size_t)L.n_part * (2 * sizeof(long long) + 2 * sizeof(double) + kMaxPorts * c));
@@ -78,17 +69,17 @@ Layout make_layout(const pngf_config& cfg) {
   L.xs = take(mixed ? (1 + n_o) * n * 8 * sizeof(float) : 0);
   L.xadd = take(mixed ? (size_t)L.R * 4 * sizeof(float) : 0);  // alpha_i of the mixed search as double-words
   const bool fp64 = cfg.precision == PNGF_FP64;
-  L.oz = take(fp64 ? factor_scratch_bytes(cfg.n_d) : mixed ? 2 * n * sizeof(int) : 0);  // mixed: the pivots
-  if (fp64) {
-    size_t im[4];
-    factor_images(cfg.n_d, im);
+  size_t im[5];
+  factor_images(cfg.n_d, im);
+  L.oz = take(fp64 ? factor_scratch_bytes(cfg.n_d) : pec ? im[4] : 2 * n * sizeof(int));
+  if (!mixed) {
     L.ozA = L.oz + im[0];
     L.ozB = L.oz + im[1];
     L.ozEa = L.oz + im[2];
     L.ozEb = L.oz + im[3];
   }
-  L.X64 = take(fp64 ? (size_t)kDelay64 * L.ldt * c : 0);
-  L.last64 = take(fp64 ? n * sizeof(int) : 0);
+  L.X64 = take(mixed ? 0 : (size_t)kDelay64 * L.ldt * c);
+  L.last64 = take(mixed ? 0 : n * sizeof(int));
   L.snapW = take(L.snapW_bytes);
   L.snapState = take(L.state_bytes + sizeof(Control));
   L.ctl = take(sizeof(Control));
@@ -283,6 +274,10 @@ pngf_status pngf_get_state(pngf_ctx* c, double* W, double* diag_W, double* e, do
   if (!c->factored) return PNGF_ENOTFACTORED;
   const size_t n = c->cfg.n_d, n_o = c->cfg.n_o, cs = sizeof(c128);
   cudaStream_t s = c->stream;
+  if (c->cfg.precision == PNGF_PEC) {
+    if (pngf_status st = pec_state(c, W, diag_W, e, T); st != PNGF_OK) return st;
+    W = diag_W = e = T = nullptr;
+  }
   if (W) {
     if (c->cfg.precision == PNGF_MIXED) return PNGF_EINVAL;
     if (cudaMemcpy2DAsync(W, n * cs, at<c128>(c, c->L.W), (size_t)c->L.ldw * cs, n * cs, n,

@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_batch_fp64_kernel(const Swe
       if (r == 0) return true;
       __syncthreads();
       fold64_digits(a.X64, ldx, s_al, a.last64, r, n, a.ozA, a.ozB, a.ozEa, a.ozEb, warp, NW);
-      fold64_bases(a.W, a.ldw, a.X64, ldx, s_invd, s_hist, a.last64, r, n, tid, blockDim.x);
+      fold64_bases(a.W, a.ldw, a.X64, ldx, s_invd, s_hist, a.last64, nullptr, r, n, tid, blockDim.x);
       __syncthreads();
       const bool ok = fold64_product(oz, b_smem, a.W, a.ldw, n, r, a.ozA, a.ozB, a.ozEa, a.ozEb, 0, 1);
       for (int q = tid; q < n; q += blockDim.x) {

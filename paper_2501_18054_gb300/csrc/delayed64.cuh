@@ -70,6 +70,32 @@ __device__ __forceinline__ bool score_flip64(const ObjParams& op, c128 dv, bool 
   return true;
 }
 
+// The same for a perfect-conductor pixel (pec.cu): alpha = -1 / S_kk, and row k
+// restarts from +-i / S_kk times the column (+: metal put in).
+__device__ __forceinline__ c128 pec_rotate(c128 z, bool metal) {  // +i z or -i z
+  return metal ? mk(-z.y, z.x) : mk(z.y, -z.x);
+}
+__device__ __forceinline__ c128 pec_unrotate(c128 z, bool metal) { return pec_rotate(z, !metal); }
+template <class TRow>
+__device__ __forceinline__ bool score_pec(const ObjParams& op, bool on, c128 diag, c128 e, TRow T, const c128* o,
+                                          double& f_new, c128& alpha, c128& coef, c128& inv_d) {
+  const double d2 = cabs2(diag);
+  if (__double_as_longlong(d2) < __double_as_longlong(1e-28)) return false;
+  const double r = rcp_pos(d2);
+  const c128 sg = mk(diag.x * r, -diag.y * r);
+  alpha = mk(-sg.x, -sg.y);
+  inv_d = pec_rotate(sg, !on);
+  coef = cmul(alpha, e);
+  double f = 0.0;
+#pragma unroll 1
+  for (int p = 0; p < op.n_o; ++p) {
+    if (op.w[p] == 0.0) continue;
+    f += objective_term(op, p, cfma(coef, T(p), o[p]));
+  }
+  f_new = f;
+  return true;
+}
+
 // improvement beyond the threshold, by the sign of an FP64 difference
 __device__ __forceinline__ bool improves64(const ObjParams& op, double f_new, double f, double thr) {
   return gain_of(op, f_new, f) - thr > 0.0;
@@ -139,13 +165,16 @@ __device__ __noinline__ void fold64_digits(const c128* X, size_t ldx, const c128
 }
 
 // the restarted rows and columns of W: x_i / d_i for the last flip i of every
-// pixel in the set (hist[i]: the pixel flipped), threads gt of nt
+// pixel in the set (hist[i]: the pixel flipped), threads gt of nt.  metal (PEC):
+// the present design, whose restarted diagonal is the reciprocal pivot
 __device__ __forceinline__ void fold64_bases(c128* W, int ldw, const c128* X, size_t ldx, const c128* inv_d,
-                                             const int* hist, const int* last, int r, int n, int gt, int nt) {
+                                             const int* hist, const int* last, const uint8_t* metal, int r, int n, int gt,
+                                             int nt) {
   for (int q = gt; q < r * n; q += nt) {
     const int i = q / n, j = q - i * n, k = hist[i];
     if (last[k] != i || (j != k && last[j] > i)) continue;
-    W[j >= k ? (size_t)k * ldw + j : (size_t)j * ldw + k] = cmul(X[(size_t)i * ldx + j], inv_d[i]);
+    W[j >= k ? (size_t)k * ldw + j : (size_t)j * ldw + k] =
+        metal && j == k ? pec_unrotate(inv_d[i], metal[k] != 0) : cmul(X[(size_t)i * ldx + j], inv_d[i]);
   }
 }
 

@@ -634,12 +634,13 @@ static FactorScratch factor_scratch(int n) {
   return f;
 }
 size_t factor_scratch_bytes(int n) { return factor_scratch(n).total; }
-void factor_images(int n, size_t off[4]) {
+void factor_images(int n, size_t off[5]) {
   const FactorScratch f = factor_scratch(n);
   off[0] = f.imgA;
   off[1] = f.imgB;
   off[2] = f.ea;
   off[3] = f.eb;
+  off[4] = f.act;  // the end of the four
 }
 
 // ---------------------------------------------------------------- driver

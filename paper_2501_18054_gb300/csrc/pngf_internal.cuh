@@ -123,13 +123,13 @@ __device__ __forceinline__ void latch_status(Control* ctl, int s) {
 
 // ---------------------------------------------------------------- context
 struct Layout {
-  size_t W, LU, Q, pj, pR, pdiagH, Wlo_re, Wlo_im, X, xa, diag, e, T, v, b, pos_of, scr, part, rec, slots, actg, gsum, gsplit, xs, xadd, cbuf, rbuf,
+  size_t W, LU, Wlo_re, Wlo_im, X, xa, diag, e, T, v, b, pos_of, scr, part, rec, slots, actg, gsum, gsplit, xs, xadd, cbuf, rbuf,
       snapW, snapState, ctl, total;
   size_t snapW_bytes;  // bytes of the maintained inverse copied by snapshot
   size_t tcimg, tcimgA_bytes, tcimg_bytes;  // mixed path: operand images of the tensor-core fold
-  size_t oz;  // scratch of the factor (digit images, lists, candidate rows)
+  size_t oz;  // FP64: scratch of the factor (digit images, lists, candidate rows); mixed: its pivots; PEC: digit images
   size_t ozA, ozB, ozEa, ozEb;  // its digit images and row exponents (the folds of the FP64 search use them too)
-  size_t X64, last64;  // FP64: delayed columns (kDelay64 x ldt), index of each pixel's last flip among them
+  size_t X64, last64;  // FP64, PEC: delayed columns (kDelay64 x ldt), index of each pixel's last flip among them
   int ldw, ldl, ldt, R, n_part;
   size_t state_bytes;  // contiguous state block [diag .. b] copied by snapshot
 };
@@ -168,7 +168,7 @@ pngf_status factor_fp64(pngf_ctx* c, const uint8_t* b);
 // factor_mixed.cu
 pngf_status factor_mixed(pngf_ctx* c, const uint8_t* b);
 size_t factor_scratch_bytes(int n);
-void factor_images(int n, size_t off[4]);  // offsets of the digit images A, B and the row exponents in the scratch
+void factor_images(int n, size_t off[5]);  // offsets of the digit images A, B and the row exponents in the scratch, and their end
 // sweep_mixed.cu
 pngf_status run_sweep_mixed(pngf_ctx* c, int n_sweeps, const int32_t* order, int32_t* trace,
                             double* trace_f, int32_t trace_cap, int64_t* counters);
@@ -194,6 +194,7 @@ pngf_status run_sweep_pec(pngf_ctx* c, int n_sweeps, const int32_t* order, int32
                           int32_t trace_cap, int64_t* counters);
 pngf_status accept_flip_pec(pngf_ctx* c, int pixel);
 pngf_status score_flips_pec(pngf_ctx* c, const int32_t* pixels, int m, double* f_new);
+pngf_status pec_state(pngf_ctx* c, double* W, double* diag, double* e, double* T);
 // gradient.cu
 pngf_status gradient(pngf_ctx* c, double* grad, double* dodrho);
 // general.cu
