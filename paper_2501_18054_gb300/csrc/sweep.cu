@@ -311,37 +311,84 @@ __global__ void score_kernel(SweepArgs a, const int32_t* __restrict__ pixels, in
   }
 }
 
-// one CTA: pivot of pixel k, new o and f, column copy into cbuf, pivot record
+// ---- one kept flip.  Two launches: the pivot (formed by every block for
+// itself), the column c = W[:, k] and alpha c; then the state and W += alpha c
+// c^T on the upper triangle.
 struct PivotRecord {
   Pivot pv;
 };
 
-__global__ void accept_pivot_kernel(SweepArgs a, int k, PivotRecord* rec) {
+__global__ void __launch_bounds__(256) accept_prepare_kernel(SweepArgs a, int k, PivotRecord* rec, c128* ac) {
+  __shared__ Pivot s_pv;
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  c128 c = mk(0.0, 0.0);
+  if (j < a.n) {
+    c = j >= k ? a.W[(size_t)k * a.ldw + j] : a.W[(size_t)j * a.ldw + k];
+    a.cbuf[j] = c;
+  }
   if (threadIdx.x == 0) {
-    Pivot pv;
-    make_pivot(a, k, pv);
-    rec->pv = pv;
+    const c128 dv = a.dv[k], delta = a.b[k] ? mk(-dv.x, -dv.y) : dv, d = cfms(delta, a.diag[k], mk(1.0, 0.0));
+    const double r = rcp_pos(cabs2(d));
+    s_pv.k = k;
+    s_pv.alpha = cmul(delta, mk(d.x * r, -d.y * r));
+    s_pv.coef = cmul(s_pv.alpha, a.e[k]);
+    FOR_PORTS(p, a.n_o) s_pv.Tk[p] = a.T[(size_t)p * a.ldt + k];
+  }
+  __syncthreads();
+  if (ac && j < a.n) ac[j] = cmul(s_pv.alpha, c);
+  if (blockIdx.x == 0 && threadIdx.x == blockDim.x - 1) {
+    rec->pv = s_pv;
     c128 o[kMaxPorts];
-    FOR_PORTS(p, a.n_o) o[p] = cfma(pv.coef, pv.Tk[p], a.ctl->o[p]);
+    FOR_PORTS(p, a.n_o) o[p] = cfma(s_pv.coef, s_pv.Tk[p], a.ctl->o[p]);
     FOR_PORTS(p, a.n_o) a.ctl->o[p] = o[p];
     a.ctl->f = objective_of(a.op, o);
     a.ctl->n_acc_total += 1;
   }
 }
 
-__global__ void accept_gather_kernel(SweepArgs a, int k) {
-  int per = (a.n + gridDim.x - 1) / gridDim.x;
-  int pb = blockIdx.x * per, pe = min(a.n, pb + per);
-  gather_column(a, k, pb, pe);
-}
-
-__global__ void __launch_bounds__(kThreads) accept_update_kernel(SweepArgs a, const PivotRecord* rec) {
-  const int P = gridDim.x, cta = blockIdx.x, n = a.n;
+// A warp takes 128 columns of one row at a time: four independent 512-byte
+// reads in flight, and alpha c_i once per row piece (from `ac`, or formed here
+// where the caller has no room for it).  Bound by the FP64 pipe, one complex
+// FMA per element: 14 us at N_d = 2112, where a flip takes 32 us with its two
+// launches (about 52 with alpha c_i formed per element, in three launches).
+// 256 columns a piece: 36 us (half the CTAs fit an SM).
+constexpr int kPiece = 128;
+__global__ void __launch_bounds__(kThreads, 2) accept_update_kernel(SweepArgs a, const PivotRecord* rec, const c128* ac) {
+  const int P = gridDim.x, cta = blockIdx.x, n = a.n, lane = threadIdx.x & 31;
   const int pb = (int)((long long)n * cta / P), pe = (int)((long long)n * (cta + 1) / P);
-  const long long E = (long long)n * (n + 1) / 2;
-  Pivot pv = rec->pv;
+  const Pivot& pv = rec->pv;
+  const c128 alpha = pv.alpha;
   update_state(a, pv, pb, pe);
-  rank1_upper(a.W, n, a.ldw, a.cbuf, pv.alpha, E * cta / P, E * (cta + 1) / P);
+  // the pieces of a group of kPiece rows: C - g each, g the group
+  const int C = (n + kPiece - 1) / kPiece, nw = P * (kThreads / 32);
+  int u = cta + P * (int)(threadIdx.x >> 5), g = 0;  // neighbouring pieces on different SMs
+  while (true) {
+    while (g < C && u >= kPiece * (C - g)) {
+      u -= kPiece * (C - g);
+      ++g;
+    }
+    if (g >= C) break;
+    const int i = g * kPiece + u / (C - g), j0 = (g + u % (C - g)) * kPiece + lane;
+    if (i < n) {
+      const c128 ai = ac ? ac[i] : cmul(alpha, a.cbuf[i]);
+      c128* row = a.W + (size_t)i * a.ldw;
+      c128 w[kPiece / 32], c[kPiece / 32];
+#pragma unroll
+      for (int q = 0; q < kPiece / 32; ++q) {
+        const int j = j0 + 32 * q;
+        if (j >= i && j < n) {
+          w[q] = row[j];
+          c[q] = a.cbuf[j];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kPiece / 32; ++q) {
+        const int j = j0 + 32 * q;
+        if (j >= i && j < n) row[j] = cfma(ai, c[q], w[q]);
+      }
+    }
+    u += nw;
+  }
 }
 
 __global__ void set_wait_kernel(Control* ctl, unsigned long long polls, int hold_plus1) {
@@ -431,13 +478,19 @@ pngf_status score_flips(pngf_ctx* c, const int32_t* pixels, int m, double* f_new
   return cuda_status(cudaGetLastError());
 }
 
+static pngf_status launch_accept(pngf_ctx* c, const SweepArgs& a, int pixel, PivotRecord* rec, c128* ac) {
+  accept_prepare_kernel<<<(a.n + 255) / 256, 256, 0, c->stream>>>(a, pixel, rec, ac);
+  int blocks = (a.n + 7) / 8;  // small regions: a few rows' work per CTA
+  if (blocks > 2 * c->n_sm) blocks = 2 * c->n_sm;
+  accept_update_kernel<<<blocks, kThreads, 0, c->stream>>>(a, rec, ac);
+  return cuda_status(cudaGetLastError());
+}
+
 pngf_status accept_flip(pngf_ctx* c, int pixel) {
   SweepArgs a = make_args(c);
-  PivotRecord* rec = reinterpret_cast<PivotRecord*>(a.rbuf);  // scratch
-  accept_pivot_kernel<<<1, 32, 0, c->stream>>>(a, pixel, rec);
-  accept_gather_kernel<<<c->n_sm, 256, 0, c->stream>>>(a, pixel);
-  accept_update_kernel<<<c->n_sm * 2, kThreads, 0, c->stream>>>(a, rec);
-  return cuda_status(cudaGetLastError());
+  PivotRecord* rec = reinterpret_cast<PivotRecord*>(a.rbuf);        // scratch: block 0 of the refresh vectors
+  c128* ac = a.rbuf + (size_t)3 * (1 + a.n_o) * a.n + sizeof(PivotRecord) / sizeof(c128) + 1;  // past the record
+  return launch_accept(c, a, pixel, rec, ac);
 }
 
 // ---------------------------------------------------------------- accept without workspace scratch
@@ -478,10 +531,7 @@ pngf_status accept_flip_noalloc(pngf_ctx* c, int pixel) {
   SweepArgs a = make_args(c);
   PivotRecord* rec = static_cast<PivotRecord*>(base);
   a.cbuf = reinterpret_cast<c128*>(static_cast<unsigned char*>(base) + kNoAllocRecordBytes);
-  accept_pivot_kernel<<<1, 32, 0, c->stream>>>(a, pixel, rec);
-  accept_gather_kernel<<<c->n_sm, 256, 0, c->stream>>>(a, pixel);
-  accept_update_kernel<<<c->n_sm * 2, kThreads, 0, c->stream>>>(a, rec);
-  return cuda_status(cudaGetLastError());
+  return launch_accept(c, a, pixel, rec, nullptr);
 }
 
 }  // namespace pngf

@@ -256,9 +256,7 @@ __device__ __forceinline__ void tri_rc(long long e, int n, int& i, int& j) {
   j = lo + (int)(e - ((long long)lo * n - (long long)lo * (lo - 1) / 2));
 }
 
-// W += alpha c c^T on packed elements [eb, ee) of the upper triangle.
-// Thread t walks elements eb + t + m*blockDim; four consecutive steps of the
-// walk are issued together so that four independent loads are in flight.
+// the walk of a thread over packed elements of the upper triangle, `stride` at a time
 __device__ __forceinline__ void tri_step(int& i, int& j, int n, int stride) {
   j += stride;
   // carry into the following rows (row i+1 starts at column i+1); past the
@@ -267,46 +265,6 @@ __device__ __forceinline__ void tri_step(int& i, int& j, int n, int stride) {
     j -= n;
     ++i;
     j += i;
-  }
-}
-
-__device__ void rank1_upper(c128* __restrict__ W, int n, int ldw, const c128* __restrict__ c, c128 alpha,
-                            long long eb, long long ee) {
-  long long e = eb + threadIdx.x;
-  if (e >= ee) return;
-  const int stride = blockDim.x;
-  int i0, j0;
-  tri_rc(e, n, i0, j0);
-  while (e + 3LL * stride < ee) {
-    int i1 = i0, j1 = j0;
-    tri_step(i1, j1, n, stride);
-    int i2 = i1, j2 = j1;
-    tri_step(i2, j2, n, stride);
-    int i3 = i2, j3 = j2;
-    tri_step(i3, j3, n, stride);
-    c128* p0 = W + (size_t)i0 * ldw + j0;
-    c128* p1 = W + (size_t)i1 * ldw + j1;
-    c128* p2 = W + (size_t)i2 * ldw + j2;
-    c128* p3 = W + (size_t)i3 * ldw + j3;
-    c128 w0 = *p0, w1 = *p1, w2 = *p2, w3 = *p3;
-    c128 c0 = c[j0], c1 = c[j1], c2 = c[j2], c3 = c[j3];
-    c128 a0 = cmul(alpha, c[i0]);
-    c128 a1 = (i1 == i0) ? a0 : cmul(alpha, c[i1]);
-    c128 a2 = (i2 == i1) ? a1 : cmul(alpha, c[i2]);
-    c128 a3 = (i3 == i2) ? a2 : cmul(alpha, c[i3]);
-    *p0 = cfma(a0, c0, w0);
-    *p1 = cfma(a1, c1, w1);
-    *p2 = cfma(a2, c2, w2);
-    *p3 = cfma(a3, c3, w3);
-    i0 = i3;
-    j0 = j3;
-    tri_step(i0, j0, n, stride);
-    e += 4LL * stride;
-  }
-  for (; e < ee; e += stride) {
-    c128* p = W + (size_t)i0 * ldw + j0;
-    *p = cfma(cmul(alpha, c[i0]), c[j0], *p);
-    tri_step(i0, j0, n, stride);
   }
 }
 
@@ -344,12 +302,6 @@ __device__ void update_state(const SweepArgs& a, const Pivot& pv, int pb, int pe
       a.v[j] = nb ? a.dv[j] : mk(0.0, 0.0);
     }
   }
-}
-
-// c_j = W[k][j] (j >= k) or W[j][k] (j < k) for j in [pb, pe)
-__device__ void gather_column(const SweepArgs& a, int k, int pb, int pe) {
-  for (int j = pb + threadIdx.x; j < pe; j += blockDim.x)
-    a.cbuf[j] = (j >= k) ? a.W[(size_t)k * a.ldw + j] : a.W[(size_t)j * a.ldw + k];
 }
 
 // ---------------------------------------------------------------- refresh
