@@ -71,7 +71,7 @@ Layout make_layout(const pngf_config& cfg) {
   const bool fp64 = cfg.precision == PNGF_FP64;
   size_t im[5];
   factor_images(cfg.n_d, im);
-  L.oz = take(fp64 ? factor_scratch_bytes(cfg.n_d) : pec ? im[4] : 2 * n * sizeof(int));
+  L.oz = take(pec ? im[4] : factor_scratch_bytes(cfg.n_d, fp64));
   if (!mixed) {
     L.ozA = L.oz + im[0];
     L.ozB = L.oz + im[1];

@@ -35,16 +35,6 @@ namespace {
 constexpr int kDelay64 = OZ_KMAX;  // columns held; one exact accumulation of the fold
 constexpr int kChains64 = 8;       // chains of the column sum
 
-// 1 / x for x > 0: FP32 seed and two Newton steps (2^-22, 2^-44, 2^-88), no
-// FP64 division (ten instructions' time on the FP64 pipe)
-__device__ __forceinline__ double rcp_pos(double x) {
-  const int ex = oz_exp(x);
-  if (ex < 1023 - 120 || ex > 1023 + 120) return 1.0 / x;
-  double r = (double)(1.0f / (float)x);
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
-}
-
 // Candidate flip of a pixel (Eq. 14): inv_d = 1 / d, d = 1 - delta W_kk, alpha =
 // delta / d, coef = alpha e_k and the objective of o + coef T[:, k]; T(p) is row p of T at
 // the pixel.  False for a singular candidate (|d| < 1e-14).  Ports of weight

@@ -27,71 +27,17 @@
 // digits 2.5.
 #include <cstdio>
 
+#include "factor_common.cuh"
 #include "form_ports.cuh"
 #include "ozaki.cuh"
 
 namespace pngf {
 namespace {
 
-constexpr int NB = 32;        // panel width
 constexpr int BB = 64;        // block of the substitutions, K of their products
 constexpr int FT_THREADS = OZ_THREADS;
 constexpr int FT_WARPS = FT_THREADS / 32;
 
-struct FactorArgs {
-  int n, n_o, ldw, ldt;
-  const c128* G;
-  const c128* God;
-  const c128* cd;
-  const c128* dv;
-  const uint8_t* b_in;
-  c128* LU;  // M_aa, m x m, leading dimension ldw
-  c128* W;   // n x ldw, column n holds e
-  c128* T;
-  c128* v;
-  uint8_t* b;
-  c128* diag;
-  c128* e;
-  double* Gs;  // Re G + Im G
-  int* act;    // the m pixels that are on, ascending, then the n - m others
-  int* count;  // m
-  unsigned char* imgA;
-  unsigned char* imgB;
-  int* ea;
-  int* eb;
-  c128* cand;               // [2][P][NB] candidate pivot rows
-  unsigned long long* key;  // [2][P] their keys
-  int* cand_row;            // [2][P]
-  c128* drow;               // [2][NB] diagonal row of the column
-  int* piv;                 // NB pivots of the panel
-  c128* dinv;               // n reciprocals of the pivots
-  int* perm;                // row i of the pivoted M_aa is row perm[i] of M_aa
-  c128* binv;               // inverses of the BB x BB diagonal blocks: of L, then of U
-  Control* ctl;
-};
-
-// |re| + |im| as an order-preserving key (NaN lowest: it is taken only where
-// nothing else is left)
-__device__ __forceinline__ unsigned long long pivot_key(c128 z) {
-  const double a = cabs1(z);
-  return isnan(a) ? 0ull : (unsigned long long)__double_as_longlong(a);
-}
-
-// 1 / z without FP64 divisions (each occupies the FP64 pipe for ten
-// instructions): z is scaled by a power of two to [1, 2), |z|^-2 by an FP32
-// seed and three Newton steps (quadratic: 2^-22, 2^-44, 2^-88)
-__device__ __forceinline__ c128 crecip(c128 z) {
-  const int ex = max(oz_exp(z.x), oz_exp(z.y));
-  if (ex < 64 || ex > 1980) return cdiv(mk(1.0, 0.0), z);  // zero, tiny, huge, infinite, NaN
-  const double sc = __longlong_as_double((long long)(2046 - ex) << 52);  // 2^(1023 - ex)
-  const double x = z.x * sc, y = z.y * sc;
-  const double d = fma(x, x, y * y);  // in [1, 8)
-  double r = (double)(1.0f / (float)d);
-  r = fma(r, fma(-d, r, 1.0), r);
-  r = fma(r, fma(-d, r, 1.0), r);
-  r *= sc;
-  return mk(x * r, -y * r);
-}
 
 // the ascending lists of the pixels that are on and off (one CTA)
 __device__ void factor_lists(const FactorArgs& a) {
@@ -119,167 +65,6 @@ __device__ void factor_lists(const FactorArgs& a) {
     else a.act[off_++] = i;
   }
   if (threadIdx.x == 0) *a.count = m;
-}
-
-// ---------------------------------------------------------------- panel
-// LU of rows [j0, m) x columns [j0, j0 + jb) with partial pivoting (|re| + |im|,
-// ties -> lowest row).  CTA q holds its chunk of the rows in shared memory.
-// Per column: every CTA publishes its candidate row (and the owner the
-// diagonal row), one grid barrier, every CTA picks the winner, swaps what it
-// owns and updates its rows, tracking the next column's candidate.  The rows
-// travel with the candidates, so one barrier per column is enough.
-__device__ bool factor_panel(const FactorArgs& a, int m, int j0, int jb, c128* ps) {
-  __shared__ unsigned long long s_key[FT_WARPS];
-  __shared__ int s_row[FT_WARPS];
-  __shared__ c128 s_u[NB], s_d[NB];
-  __shared__ c128 s_inv;
-  __shared__ int s_p;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, P = gridDim.x, cta = blockIdx.x;
-  const int rows = m - j0;
-  const int rb = j0 + (int)((long long)rows * cta / P), re = j0 + (int)((long long)rows * (cta + 1) / P);
-  const bool act_lane = lane < jb;
-  unsigned long long bk = 0;
-  int br = 0x7fffffff;
-  for (int r = rb + warp; r < re; r += FT_WARPS) {
-    const c128 z = act_lane ? a.LU[(size_t)r * a.ldw + j0 + lane] : mk(0.0, 0.0);
-    ps[(r - rb) * NB + lane] = z;
-    if (lane == 0) {
-      const unsigned long long k = pivot_key(z);
-      if (br == 0x7fffffff || k > bk) { bk = k; br = r; }
-    }
-  }
-  for (int jj = 0; jj < jb; ++jj) {
-    const int col = j0 + jj, par = jj & 1;
-    // ---- this CTA's candidate (held by lane jj of every warp)
-    bk = __shfl_sync(0xffffffffu, bk, jj);
-    br = __shfl_sync(0xffffffffu, br, jj);
-    if (lane == 0) { s_key[warp] = bk; s_row[warp] = br; }
-    __syncthreads();
-    if (warp == 0) {
-      unsigned long long k = lane < FT_WARPS ? s_key[lane] : 0ull;
-      int r = lane < FT_WARPS ? s_row[lane] : 0x7fffffff;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const unsigned long long ok = __shfl_xor_sync(0xffffffffu, k, off);
-        const int orr = __shfl_xor_sync(0xffffffffu, r, off);
-        if (ok > k || (ok == k && orr < r)) { k = ok; r = orr; }
-      }
-      if (r != 0x7fffffff) a.cand[((size_t)par * P + cta) * NB + lane] = ps[(r - rb) * NB + lane];
-      if (lane == 0) {
-        a.key[par * P + cta] = k;
-        a.cand_row[par * P + cta] = r;
-      }
-    } else if (warp == 1 && col >= rb && col < re) {
-      a.drow[par * NB + lane] = ps[(col - rb) * NB + lane];
-    }
-    if (!grid_sync(a.ctl)) return false;
-    // ---- the pivot, its row and its reciprocal (warp 0), the diagonal row (warp 1)
-    if (warp == 0) {
-      unsigned long long k = 0;
-      int r = 0x7fffffff, q = -1;
-      for (int c = lane; c < P; c += 32) {
-        const unsigned long long ck = a.key[par * P + c];
-        const int cr = a.cand_row[par * P + c];
-        if (ck > k || (ck == k && cr < r)) { k = ck; r = cr; q = c; }
-      }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const unsigned long long ok = __shfl_xor_sync(0xffffffffu, k, off);
-        const int orr = __shfl_xor_sync(0xffffffffu, r, off), oq = __shfl_xor_sync(0xffffffffu, q, off);
-        if (ok > k || (ok == k && orr < r)) { k = ok; r = orr; q = oq; }
-      }
-      const bool singular = k == 0;  // an exactly zero (or NaN) column: keep the diagonal row
-      const c128 u = singular ? a.drow[par * NB + lane] : a.cand[((size_t)par * P + q) * NB + lane];
-      s_u[lane] = u;
-      const c128 pv = mk(__shfl_sync(0xffffffffu, u.x, jj), __shfl_sync(0xffffffffu, u.y, jj));
-      const c128 inv = crecip(pv);
-      if (lane == 0) {
-        s_inv = inv;
-        s_p = singular ? col : r;
-        if (cta == 0) {
-          a.piv[jj] = s_p;
-          a.dinv[col] = inv;
-          if (singular) latch_status(a.ctl, PNGF_ESINGULAR);
-        }
-      }
-    } else if (warp == 1) {
-      s_d[lane] = a.drow[par * NB + lane];
-    }
-    __syncthreads();
-    const int p = s_p;
-    if (warp == 0 && p != col && p >= rb && p < re) ps[(p - rb) * NB + lane] = s_d[lane];
-    if (warp == 1 && col >= rb && col < re) ps[(col - rb) * NB + lane] = s_u[lane];
-    __syncthreads();
-    // ---- scale the column, update the rest of the panel (lane = column)
-    const c128 inv = s_inv, u = s_u[lane];
-    bk = 0;
-    br = 0x7fffffff;
-    for (int r = max(rb, col + 1) + warp; r < re; r += FT_WARPS) {
-      c128* row = ps + (r - rb) * NB;
-      const c128 z = row[lane];
-      const c128 l = cmul(row[jj], inv);
-      __syncwarp();  // every lane has read row[jj]
-      if (lane == jj) {
-        row[lane] = l;
-      } else if (lane > jj && act_lane) {
-        const c128 nz = cfms(l, u, z);
-        row[lane] = nz;
-        if (lane == jj + 1) {
-          const unsigned long long k = pivot_key(nz);
-          if (br == 0x7fffffff || k > bk) { bk = k; br = r; }
-        }
-      }
-      __syncwarp();
-    }
-    // lane jj + 1 holds the next candidate; the next iteration's shuffle takes it from there
-    if (jj + 1 < jb) {
-      bk = __shfl_sync(0xffffffffu, bk, jj + 1);
-      br = __shfl_sync(0xffffffffu, br, jj + 1);
-    }
-  }
-  __syncthreads();
-  for (int r = rb + warp; r < re; r += FT_WARPS)
-    if (act_lane) a.LU[(size_t)r * a.ldw + j0 + lane] = ps[(r - rb) * NB + lane];
-  return grid_sync(a.ctl);
-}
-
-// ---------------------------------------------------------------- interchanges
-// Net effect of the panel's interchanges, formed by warp 0 of every CTA: the
-// row top_src[i] moves to row j0 + i, and row ext_src[e] to the row
-// ext_row[e] below the panel's block (e < n_ext <= NB).
-struct Swaps {
-  int top_src[NB], ext_row[NB], ext_src[NB], n_ext;
-};
-
-__device__ __forceinline__ void net_swaps(const FactorArgs& a, int j0, int jb, Swaps& sw) {
-  if (threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
-  int top = j0 + lane, er = -1, es = -1, ne = 0;
-  const int pl = lane < jb ? a.piv[lane] : -1;
-  for (int jj = 0; jj < jb; ++jj) {
-    const int p = __shfl_sync(0xffffffffu, pl, jj);
-    const int tj = __shfl_sync(0xffffffffu, top, jj);
-    if (p < j0 + jb) {
-      const int tp = __shfl_sync(0xffffffffu, top, p - j0);
-      if (lane == jj) top = tp;
-      if (lane == p - j0) top = tj;
-    } else {
-      const unsigned hit = __ballot_sync(0xffffffffu, er == p);
-      const int s = hit ? __ffs(hit) - 1 : ne++;
-      if (!hit && lane == s) { er = p; es = p; }
-      const int v = __shfl_sync(0xffffffffu, es, s);
-      if (lane == jj) top = v;
-      if (lane == s) es = tj;
-    }
-  }
-  sw.top_src[lane] = top;
-  sw.ext_row[lane] = er;
-  sw.ext_src[lane] = es;
-  if (lane == 0) sw.n_ext = ne;
-}
-
-__device__ __forceinline__ c128 shfl_c(c128 z, int src) {
-  return mk(__shfl_sync(0xffffffffu, z.x, src), __shfl_sync(0xffffffffu, z.y, src));
 }
 
 // ---------------------------------------------------------------- diagonal blocks
@@ -332,9 +117,23 @@ __device__ void block_inverse(const FactorArgs& a, int m, int bi, int upper, int
   }
 }
 
+// Whether a pixel that is on has |dv G_kk| >= 16: lossy metal (500) and the
+// like, against 0.5 for eps = 10.  Such systems go to factor_pipe.cu.  The
+// elimination here is as accurate, but what a search reports there can hang on
+// the last bits of the start state (a metal-filled guide transmits 10^-9 of the
+// power: rounding of 10^-14 in the fields is 10^-9 of it), and stays the same.
+__global__ void contrast_kernel(const c128* G, const c128* dv, const uint8_t* b, int n, int* high) {
+  int h = 0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x)
+    if (b[i] && cabs2(dv[i]) * cabs2(G[(size_t)i * n + i]) >= 256.0) h = 1;
+  h = __syncthreads_or(h);
+  if (threadIdx.x == 0) *high = h;
+}
+
 // ---------------------------------------------------------------- the factorisation
 __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_constant__ FactorArgs a) {
   extern __shared__ __align__(128) unsigned char f_smem[];
+  if (*a.high) return;
   __shared__ __align__(8) unsigned long long s_bars[OZ_NBAR];
   __shared__ unsigned s_tmem;
   __shared__ Swaps s_sw;
@@ -406,7 +205,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
   // ---- LU
   for (int j0 = 0; ok && j0 < m; j0 += NB) {
     const int jb = min(NB, m - j0), i1 = j0 + jb, rest = m - i1, nk = (jb + OZ_KC - 1) / OZ_KC;
-    ok = factor_panel(a, m, j0, jb, sm);
+    ok = factor_panel<FT_WARPS, false>(a, m, j0, jb, sm);
     if (!ok) break;
     net_swaps(a, j0, jb, s_sw);
     // L of the block (unit lower), column-major: Ls[k][row]
@@ -415,54 +214,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
       sm[q] = (r < jb && k < r) ? a.LU[(size_t)(j0 + r) * ldw + j0 + k] : mk(0.0, 0.0);
     }
     __syncthreads();
-    // interchanges of the other columns, and L^-1 on those right of the panel:
-    // one warp per two columns, lane = row (a warp's FP64 instruction costs
-    // the same for one lane as for 32)
-    {
-      const int ur = (rest + 1) / 2, ul = j0 / 2;
-      const int ts = s_sw.top_src[lane], er = s_sw.ext_row[lane], es = s_sw.ext_src[lane];
-      for (int u = gw; u < ur + ul; u += nw) {
-        const bool left = u >= ur;
-        const int c = left ? 2 * (u - ur) : i1 + 2 * u;
-        const bool two = c + 1 < (left ? j0 : m);
-        c128* base = a.LU + c;
-        c128 x0 = mk(0.0, 0.0), x1 = x0, y0 = x0, y1 = x0;
-        if (lane < jb) {
-          const c128* p = base + (size_t)ts * ldw;
-          x0 = p[0];
-          if (two) x1 = p[1];
-        }
-        if (er >= 0) {
-          const c128* p = base + (size_t)es * ldw;
-          y0 = p[0];
-          if (two) y1 = p[1];
-        }
-        __syncwarp();
-        if (er >= 0) {
-          c128* p = base + (size_t)er * ldw;
-          p[0] = y0;
-          if (two) p[1] = y1;
-        }
-        if (!left)
-          for (int k = 0; k + 1 < jb; ++k) {
-            const c128 l = sm[k * NB + lane];  // zero for row <= k
-            const c128 a0 = shfl_c(x0, k), a1 = shfl_c(x1, k);
-            x0 = cfms(l, a0, x0);
-            x1 = cfms(l, a1, x1);
-          }
-        if (lane < jb) {
-          c128* p = base + (size_t)(j0 + lane) * ldw;
-          p[0] = x0;
-          if (two) p[1] = x1;
-        }
-      }
-      if (cta == P - 1 && warp == FT_WARPS - 1) {  // the row permutation
-        const int x = lane < jb ? a.perm[ts] : 0, y = er >= 0 ? a.perm[es] : 0;
-        __syncwarp();
-        if (lane < jb) a.perm[j0 + lane] = x;
-        if (er >= 0) a.perm[er] = y;
-      }
-    }
+    swap_and_solve(a, s_sw, sm, m, j0, jb, gw, nw);
     if (rest > 0) digits_A(rest, jb, [&](int r, int k) { return a.LU[(size_t)(i1 + r) * ldw + j0 + k]; });
     if (!(ok = images_done())) break;
     if (rest == 0) continue;
@@ -604,12 +356,12 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
 
 }  // namespace
 
-// bytes of the factor's scratch (c->L.oz): digit images, row exponents, lists,
-// candidate rows, reciprocals of the pivots
+// the factor's scratch (c->L.oz): digit images (not for mixed contexts), row
+// exponents, lists, candidate rows, reciprocals of the pivots
 struct FactorScratch {
-  size_t imgA, imgB, ea, eb, act, cand, key, cand_row, drow, piv, dinv, perm, binv, total;
+  size_t imgA, imgB, ea, eb, act, cand, key, cand_row, drow, piv, dinv, perm, binv, high, total;
 };
-static FactorScratch factor_scratch(int n) {
+static FactorScratch factor_scratch(int n, bool images) {
   FactorScratch f{};
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -617,10 +369,10 @@ static FactorScratch factor_scratch(int n) {
     off += (bytes + 255) / 256 * 256;
     return o;
   };
-  f.imgA = take(oz_a_bytes(n + kMaxPorts, OZ_KMAX));
-  f.imgB = take(oz_b_bytes(n + 1, OZ_KMAX));
-  f.ea = take(((size_t)n + kMaxPorts + OZ_M) * sizeof(int));
-  f.eb = take(((size_t)n + 1 + OZ_N) * sizeof(int));
+  f.imgA = take(images ? oz_a_bytes(n + kMaxPorts, OZ_KMAX) : 0);
+  f.imgB = take(images ? oz_b_bytes(n + 1, OZ_KMAX) : 0);
+  f.ea = take(images ? ((size_t)n + kMaxPorts + OZ_M) * sizeof(int) : 0);
+  f.eb = take(images ? ((size_t)n + 1 + OZ_N) * sizeof(int) : 0);
   f.act = take(((size_t)n + 64) * sizeof(int));
   f.cand = take((size_t)2 * 1024 * NB * sizeof(c128));
   f.key = take((size_t)2 * 1024 * sizeof(unsigned long long));
@@ -629,13 +381,14 @@ static FactorScratch factor_scratch(int n) {
   f.piv = take(NB * sizeof(int));
   f.dinv = take((size_t)n * sizeof(c128));
   f.perm = take((size_t)n * sizeof(int));
-  f.binv = take((size_t)2 * ((n + BB - 1) / BB) * BB * BB * sizeof(c128));
+  f.binv = take(images ? (size_t)2 * ((n + BB - 1) / BB) * BB * BB * sizeof(c128) : 0);
+  f.high = take(sizeof(int));
   f.total = off;
   return f;
 }
-size_t factor_scratch_bytes(int n) { return factor_scratch(n).total; }
+size_t factor_scratch_bytes(int n, bool images) { return factor_scratch(n, images).total; }
 void factor_images(int n, size_t off[5]) {
-  const FactorScratch f = factor_scratch(n);
+  const FactorScratch f = factor_scratch(n, true);
   off[0] = f.imgA;
   off[1] = f.imgB;
   off[2] = f.ea;
@@ -644,10 +397,10 @@ void factor_images(int n, size_t off[5]) {
 }
 
 // ---------------------------------------------------------------- driver
-pngf_status factor_fp64(pngf_ctx* c, const uint8_t* b) {
+// arguments of both factorisations
+FactorArgs factor_args(pngf_ctx* c, const uint8_t* b) {
   const int n = c->cfg.n_d;
-  cudaStream_t s = c->stream;
-  const FactorScratch f = factor_scratch(n);
+  const FactorScratch f = factor_scratch(n, c->cfg.precision == PNGF_FP64);
   char* ws = c->ws + c->L.oz;
   FactorArgs a{};
   a.n = n;
@@ -681,7 +434,16 @@ pngf_status factor_fp64(pngf_ctx* c, const uint8_t* b) {
   a.dinv = reinterpret_cast<c128*>(ws + f.dinv);
   a.perm = reinterpret_cast<int*>(ws + f.perm);
   a.binv = reinterpret_cast<c128*>(ws + f.binv);
+  a.high = reinterpret_cast<int*>(ws + f.high);
   a.ctl = at<Control>(c, c->L.ctl);
+  return a;
+}
+
+pngf_status factor_fp64(pngf_ctx* c, const uint8_t* b) {
+  const int n = c->cfg.n_d;
+  cudaStream_t s = c->stream;
+  FactorArgs a = factor_args(c, b);
+  contrast_kernel<<<1, 1024, 0, s>>>(a.G, a.dv, b, n, const_cast<int*>(a.high));
   if (cudaFuncSetAttribute(factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM) != cudaSuccess)
     return PNGF_ECUDA;
   int P = (n + 15) / 16;
@@ -691,7 +453,18 @@ pngf_status factor_fp64(pngf_ctx* c, const uint8_t* b) {
   if (cudaLaunchCooperativeKernel((const void*)factor_kernel, dim3(P), dim3(FT_THREADS), params, OZ_SMEM, s) !=
       cudaSuccess)
     return PNGF_ECUDA;
+  const pngf_status st = factor_pipe(c, a);  // the high contrast
+  if (st != PNGF_OK) return st;
   form_o<<<1, 256, 0, s>>>(c->God, c->co, a.v, a.e, n, c->obj, a.ctl);
+  return cuda_status(cudaGetLastError());
+}
+
+pngf_status factor_mixed(pngf_ctx* c, const uint8_t* b) {
+  FactorArgs a = factor_args(c, b);
+  a.high = nullptr;
+  const pngf_status st = factor_pipe(c, a);
+  if (st != PNGF_OK) return st;
+  form_o<<<1, 256, 0, c->stream>>>(c->God, c->co, a.v, a.e, a.n, c->obj, a.ctl);
   return cuda_status(cudaGetLastError());
 }
 

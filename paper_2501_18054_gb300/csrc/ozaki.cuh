@@ -38,6 +38,7 @@
 #pragma once
 
 #include "flush_tc.cuh"
+#include "fp64_fast.cuh"
 
 namespace pngf {
 namespace {
@@ -74,8 +75,6 @@ __host__ __device__ __forceinline__ size_t oz_b_bytes(int rows, int K) {
 }
 
 // ---------------------------------------------------------------- digits
-__device__ __forceinline__ int oz_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-
 // X = rint(x 2^(54 - e)), e = emax - 1022 (biased exponent emax of the row's
 // largest entry), plus the offset that turns its base-256 digits into bytes:
 // byte 6 - s of the result is digit s + 128.  Integer arithmetic only.

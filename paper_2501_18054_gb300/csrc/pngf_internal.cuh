@@ -127,7 +127,7 @@ struct Layout {
       snapW, snapState, ctl, total;
   size_t snapW_bytes;  // bytes of the maintained inverse copied by snapshot
   size_t tcimg, tcimgA_bytes, tcimg_bytes;  // mixed path: operand images of the tensor-core fold
-  size_t oz;  // FP64: scratch of the factor (digit images, lists, candidate rows); mixed: its pivots; PEC: digit images
+  size_t oz;  // FP64: scratch of the factor (digit images, lists, candidate rows); mixed: without digit images; PEC: digit images
   size_t ozA, ozB, ozEa, ozEb;  // its digit images and row exponents (the folds of the FP64 search use them too)
   size_t X64, last64;  // FP64, PEC: delayed columns (kDelay64 x ldt), index of each pixel's last flip among them
   int ldw, ldl, ldt, R, n_part;
@@ -165,9 +165,8 @@ __host__ __forceinline__ T* at(pngf_ctx* c, size_t off) {
 
 // factor.cu
 pngf_status factor_fp64(pngf_ctx* c, const uint8_t* b);
-// factor_mixed.cu
 pngf_status factor_mixed(pngf_ctx* c, const uint8_t* b);
-size_t factor_scratch_bytes(int n);
+size_t factor_scratch_bytes(int n, bool images);
 void factor_images(int n, size_t off[5]);  // offsets of the digit images A, B and the row exponents in the scratch, and their end
 // sweep_mixed.cu
 pngf_status run_sweep_mixed(pngf_ctx* c, int n_sweeps, const int32_t* order, int32_t* trace,
