@@ -26,9 +26,16 @@
 // upper triangle of every system's W (rank-m update).  Three grid barriers
 // per kept flip: after the selection, after the gather of U and V, after the
 // update (the next scores read W_KK, e_K and T[:, K] of any CTA's pixels).
+//
+// A score is a chain of some 170 FP64 instructions (64 cycles each on their
+// sub-partition), so the systems of a tile are scored, and its pivots formed, on
+// neighbouring warps; reciprocals take no FP64 division.  The rank-m update is
+// bound by the FP64 pipe (m complex FMAs per entry).  Three systems of 1024
+// pixels, 2 x 2 tiles, four sweeps: 13.9 -> 8.6 ms (before: systems one after
+// another on one warp, and one entry at a time in the update).
 #include <cstdio>
 
-#include "sweep_common.cuh"
+#include "fp64_fast.cuh"
 
 namespace pngf {
 namespace {
@@ -45,8 +52,8 @@ struct GenArgs {
   int n_sys, combine, kind;
   const int* tiles;  // n_tiles x tile_m, -1 pads
   int n_tiles, tile_m;
-  c128* U;  // [n_sys][n][tile_m]
-  c128* V;  // [n_sys][n][tile_m]
+  c128* U;  // [n_sys][tile_m][n]
+  c128* V;  // [n_sys][tile_m][n]
   int* pos_of;  // n_tiles
   double* part_gain;  // [2][P]
   long long* part_key;
@@ -98,14 +105,22 @@ __device__ __forceinline__ int tile_pixels(const GenArgs& g, int t, int n, int& 
 __device__ bool warp_gauss_jordan(c128* A, int ld, int m, int ncols) {
   const int lane = threadIdx.x & 31;
   for (int c = 0; c < m; ++c) {
-    double mag = (lane >= c && lane < m) ? cabs2(A[lane * ld + c]) : -1.0;
+    // squared magnitudes compare as integers (0: not a candidate row, or NaN)
+    unsigned long long mag = 0;
+    if (lane >= c && lane < m) {
+      const double a2 = cabs2(A[lane * ld + c]);
+      mag = oz_exp(a2) == 0x7ff ? (isinf(a2) ? (unsigned long long)__double_as_longlong(a2) : 0ull)
+                                : (unsigned long long)__double_as_longlong(a2);
+    }
     int piv = lane;
-    for (int off = 16; off > 0; off >>= 1) {
-      const double om = __shfl_xor_sync(0xffffffffu, mag, off);
+    for (int off = 8; off > 0; off >>= 1) {  // m <= 16 rows
+      const unsigned long long om = __shfl_xor_sync(0xffffffffu, mag, off);
       const int op = __shfl_xor_sync(0xffffffffu, piv, off);
       if (om > mag || (om == mag && op < piv)) { mag = om; piv = op; }
     }
-    if (!(mag >= 1e-28)) return false;
+    mag = __shfl_sync(0xffffffffu, mag, 0);
+    piv = __shfl_sync(0xffffffffu, piv, 0);
+    if (mag < (unsigned long long)__double_as_longlong(1e-28)) return false;
     if (piv != c)
       for (int j = lane; j < ncols; j += 32) {
         const c128 t = A[c * ld + j];
@@ -113,7 +128,7 @@ __device__ bool warp_gauss_jordan(c128* A, int ld, int m, int ncols) {
         A[piv * ld + j] = t;
       }
     __syncwarp();
-    const c128 inv = cdiv(mk(1.0, 0.0), A[c * ld + c]);
+    const c128 inv = crecip(A[c * ld + c]);
     __syncwarp();
     for (int j = lane; j < ncols; j += 32) A[c * ld + j] = j == c ? mk(1.0, 0.0) : cmul(A[c * ld + j], inv);
     __syncwarp();
@@ -132,11 +147,20 @@ __device__ __forceinline__ c128 delta_of(const SweepArgs& a, int k) {
   return a.b[k] ? mk(-d.x, -d.y) : d;
 }
 
+// sum over lanes 0 .. m - 1 (m <= 16; the other lanes hold zero), in every lane of the first 16
+__device__ __forceinline__ c128 tile_sum(c128 v, int m) {
+  for (int off = 1; off < m; off <<= 1) {
+    v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
+    v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
+  }
+  return mk(__shfl_sync(0xffffffffu, v.x, 0), __shfl_sync(0xffffffffu, v.y, 0));
+}
+
 // Score one tile in one system (one warp): f after the flip, or false if the
 // capacitance system is singular.  o: the system's current ports; buf: the
 // warp's kTileMax x kScoreLd scratch.
 __device__ bool score_tile_sys(const SweepArgs& a, const ObjParams& op, const c128* o, int px, int m, c128* buf,
-                               double& f_new, c128* o_new) {
+                               double& f_new) {
   const int lane = threadIdx.x & 31;
   // row `lane` of [I - D W_KK | D e_K]
   if (lane < m) {
@@ -155,11 +179,9 @@ __device__ bool score_tile_sys(const SweepArgs& a, const ObjParams& op, const c1
   double f = 0.0;
 #pragma unroll 1
   for (int p = 0; p < a.n_o; ++p) {
-    c128 t = lane < m ? cmul(a.T[(size_t)p * a.ldt + px], y) : mk(0.0, 0.0);
-    t = warp_sum(t);  // every lane holds the sum
-    const c128 on = cadd(o[p], t);
-    if (o_new) o_new[p] = on;
-    f += objective_term(op, p, on);
+    if (op.w[p] == 0.0) continue;  // adds nothing to the objective
+    const c128 t = tile_sum(lane < m ? cmul(a.T[(size_t)p * a.ldt + px], y) : mk(0.0, 0.0), m);
+    f += objective_term(op, p, cadd(o[p], t));
   }
   f_new = f;
   __syncwarp();
@@ -192,6 +214,15 @@ __device__ bool score_pixel_tile(const GenArgs& g, const c128 (*s_o)[kMaxPorts],
   return true;
 }
 
+// the same for one of the systems
+__device__ bool score_tile_of(const GenArgs& g, const c128 (*s_o)[kMaxPorts], int t, int sy, c128* buf, double& f) {
+  int m;
+  bool bad;
+  const int px = tile_pixels(g, t, g.sys[0].n, m, bad);
+  if (bad && (threadIdx.x & 31) == 0) latch_status(g.sys[0].ctl, PNGF_EINVAL);
+  return !bad && m > 0 && score_tile_sys(g.sys[sy], g.sys[sy].op, s_o[sy], px, m, buf, f);
+}
+
 // combined objective of flipping tile t (one warp); false if any system is singular
 __device__ bool score_tile(const GenArgs& g, const c128 (*s_o)[kMaxPorts], int t, c128* buf, double& F,
                            double* f_sys) {
@@ -202,7 +233,7 @@ __device__ bool score_tile(const GenArgs& g, const c128 (*s_o)[kMaxPorts], int t
   if (bad || m == 0) return false;
   double fs[kMaxSys];
   for (int s = 0; s < g.n_sys; ++s) {
-    if (!score_tile_sys(g.sys[s], g.sys[s].op, s_o[s], px, m, buf, fs[s], nullptr)) return false;
+    if (!score_tile_sys(g.sys[s], g.sys[s].op, s_o[s], px, m, buf, fs[s])) return false;
     if (f_sys) f_sys[s] = fs[s];
   }
   F = combine_of(fs, g.n_sys, g.combine, g.kind);
@@ -247,11 +278,47 @@ __device__ bool accept_pivot_sys(const SweepArgs& a, int px, int m, c128* buf, c
       if (lane < m) acc = cfma(tb, z[b * kTileMax + lane], acc);
     }
     if (lane < m) tz[p * kTileMax + lane] = acc;
-    const c128 t = warp_sum(lane < m ? cmul(tk, yi) : mk(0.0, 0.0));
+    const c128 t = tile_sum(lane < m ? cmul(tk, yi) : mk(0.0, 0.0), m);
     if (lane == 0) o[p] = cadd(o[p], t);
   }
   __syncwarp();
   return true;
+}
+
+// W[i][j] += sum_c V[c][i] U[c][j] on the upper triangle: a warp takes 128
+// columns of one row at a time, four entries a lane in flight, neighbouring
+// pieces on different SMs
+__device__ void rank_m_upper(c128* __restrict__ W, int n, int ldw, const c128* __restrict__ V,
+                             const c128* __restrict__ U, int m, int cta, int P) {
+  constexpr int kPiece = 128, kQ = kPiece / 32;
+  const int lane = threadIdx.x & 31, C = (n + kPiece - 1) / kPiece, nw = P * kWarps;
+  int u = cta + P * (int)(threadIdx.x >> 5), g = 0;
+  while (true) {
+    while (g < C && u >= kPiece * (C - g)) {  // group g: kPiece rows of C - g pieces
+      u -= kPiece * (C - g);
+      ++g;
+    }
+    if (g >= C) break;
+    const int i = g * kPiece + u / (C - g), j0 = (g + u % (C - g)) * kPiece + lane;
+    if (i < n) {
+      c128* row = W + (size_t)i * ldw;
+      c128 w[kQ];
+#pragma unroll
+      for (int q = 0; q < kQ; ++q)
+        if (j0 + 32 * q >= i && j0 + 32 * q < n) w[q] = row[j0 + 32 * q];
+      for (int c = 0; c < m; ++c) {
+        const c128 v = V[(size_t)c * n + i];
+        const c128* uc = U + (size_t)c * n;
+#pragma unroll
+        for (int q = 0; q < kQ; ++q)
+          if (j0 + 32 * q >= i && j0 + 32 * q < n) w[q] = cfma(v, uc[j0 + 32 * q], w[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < kQ; ++q)
+        if (j0 + 32 * q >= i && j0 + 32 * q < n) row[j0 + 32 * q] = w[q];
+    }
+    u += nw;
+  }
 }
 
 __global__ void __launch_bounds__(kThreads) dbs_tiles_kernel(const __grid_constant__ GenArgs g) {
@@ -260,8 +327,6 @@ __global__ void __launch_bounds__(kThreads) dbs_tiles_kernel(const __grid_consta
   const int n = g.sys[0].n, nt = g.n_tiles, M = g.tile_m;
   const int pb = (int)((long long)n * cta / P), pe = (int)((long long)n * (cta + 1) / P);
   const int tb = (int)((long long)nt * cta / P), te = (int)((long long)nt * (cta + 1) / P);
-  const long long E = (long long)n * (n + 1) / 2;
-  const long long eb = E * cta / P, ee = E * (cta + 1) / P;
   Control* ctl = g.sys[0].ctl;
   hold_if_asked(ctl);
   __shared__ c128 s_o[kMaxSys][kMaxPorts], s_o_new[kMaxSys][kMaxPorts];
@@ -272,7 +337,10 @@ __global__ void __launch_bounds__(kThreads) dbs_tiles_kernel(const __grid_consta
   __shared__ c128 s_tz[kMaxSys][kMaxPorts * kTileMax];
   __shared__ int s_px[kTileMax];
   __shared__ int s_m, s_k, s_pos, s_bad;
-  __shared__ c128 s_acc_buf[kTileMax * kAcceptLd];
+  __shared__ int s_sysbad[kMaxSys];
+  // scoring results of one round: kWarps / n_sys tiles, every system
+  __shared__ double s_fs[kWarps][kMaxSys];
+  __shared__ int s_ok[kWarps][kMaxSys];
   c128* wbuf = reinterpret_cast<c128*>(gen_smem) + (size_t)warp * kTileMax * kScoreLd;
   if (tid == 0) {
     for (int s = 0; s < g.n_sys; ++s) {
@@ -306,30 +374,55 @@ __global__ void __launch_bounds__(kThreads) dbs_tiles_kernel(const __grid_consta
     const double thr = g.tau * fmax(fabs(F), 1e-30);
     // ---- score this CTA's tiles (one warp per tile), reduce to the CTA's candidate
     if (!forced) {
-      const bool px1 = M == 1;  // single-pixel tiles: one thread per candidate
-      const int t0 = px1 ? tid : warp, ts = px1 ? (int)blockDim.x : kWarps;
-      if (g.mode == PNGF_FIRST_IMPROVEMENT) {
-        long long best = LLONG_MAX;
-        for (int ti = tb + t0; ti < te; ti += ts) {
-          const int pos = g.order ? g.pos_of[ti] : ti;
-          if (pos < t || pos >= best) continue;
-          double Fn;
-          if (!(px1 ? score_pixel_tile(g, s_o, ti, Fn) : score_tile(g, s_o, ti, wbuf, Fn, nullptr))) continue;
-          const double gain = g.kind == PNGF_OBJ_MAX_WEIGHTED_POWER ? Fn - F : F - Fn;
-          if (gain - thr > 0.0) best = pos;
+      const bool px1 = M == 1, first = g.mode == PNGF_FIRST_IMPROVEMENT;  // single-pixel tiles: one thread per candidate
+      long long best = LLONG_MAX;
+      double gb = -INFINITY;
+      int pix = INT_MAX;
+      auto consider = [&](int ti, int pos, double Fn) {
+        const double gain = g.kind == PNGF_OBJ_MAX_WEIGHTED_POWER ? Fn - F : F - Fn;
+        if (first) {
+          if (gain - thr > 0.0 && pos < best) best = pos;
+        } else if (better(gain, ti, gb, pix)) {
+          gb = gain;
+          pix = ti;
         }
-        best = block_min_ll(px1 || lane == 0 ? best : LLONG_MAX);
+      };
+      if (px1) {
+        for (int ti = tb + tid; ti < te; ti += blockDim.x) {
+          const int pos = !first ? 0 : g.order ? g.pos_of[ti] : ti;
+          double Fn;
+          if (first && (pos < t || pos >= best)) continue;
+          if (score_pixel_tile(g, s_o, ti, Fn)) consider(ti, pos, Fn);
+        }
+      } else {
+        // one warp per tile and system, the systems of a tile on neighbouring
+        // warps (different sub-partitions: a warp's FP64 chain is what a score costs)
+        const int per = kWarps / g.n_sys, slot_t = warp / g.n_sys, sy = warp % g.n_sys;
+        for (int t0 = tb; t0 < te; t0 += per) {
+          const int ti = t0 + slot_t;
+          const bool mine = slot_t < per && ti < te;
+          const int pos = mine && first ? (g.order ? g.pos_of[ti] : ti) : 0;
+          if (mine) {
+            double fv = 0.0;
+            const bool ok = (!first || pos >= t) && score_tile_of(g, s_o, ti, sy, wbuf, fv);
+            if (lane == 0) {
+              s_fs[slot_t][sy] = fv;
+              s_ok[slot_t][sy] = ok;
+            }
+          }
+          __syncthreads();
+          if (mine && sy == 0 && lane == 0) {
+            bool ok = true;
+            for (int q = 0; q < g.n_sys; ++q) ok = ok && s_ok[slot_t][q];
+            if (ok) consider(ti, pos, combine_of(s_fs[slot_t], g.n_sys, g.combine, g.kind));
+          }
+          __syncthreads();
+        }
+      }
+      if (first) {
+        best = block_min_ll(best);
         if (tid == 0) sel_offer(ctl, rd, best, cta);
       } else {
-        double gb = -INFINITY;
-        int pix = INT_MAX;
-        for (int ti = tb + t0; ti < te; ti += ts) {
-          double Fn;
-          if (!(px1 ? score_pixel_tile(g, s_o, ti, Fn) : score_tile(g, s_o, ti, wbuf, Fn, nullptr))) continue;
-          const double gain = g.kind == PNGF_OBJ_MAX_WEIGHTED_POWER ? Fn - F : F - Fn;
-          if (better(gain, ti, gb, pix)) { gb = gain; pix = ti; }
-        }
-        if (!px1 && lane != 0) { gb = -INFINITY; pix = INT_MAX; }
         block_best(gb, pix);
         if (tid == 0) {
           g.part_gain[slot * P + cta] = gb;
@@ -372,29 +465,9 @@ __global__ void __launch_bounds__(kThreads) dbs_tiles_kernel(const __grid_consta
         int m;
         bool badt;
         const int px = tile_pixels(g, k, n, m, badt);
-        if (badt || m == 0) {
-          bad = 1;
-        } else {
-          if (lane < m) s_px[lane] = px;
-          // new ports and objectives, committed only if every system's m x m system is regular
-          for (int sy = 0; sy < g.n_sys && !bad; ++sy) {
-            c128 o[kMaxPorts];
-            FOR_PORTS(p, g.sys[sy].n_o) o[p] = s_o[sy][p];
-            if (!accept_pivot_sys(g.sys[sy], px, m, s_acc_buf, s_z[sy], s_y[sy], s_tz[sy], o)) bad = 1;
-            if (lane == 0) {
-              FOR_PORTS(p, g.sys[sy].n_o) s_o_new[sy][p] = o[p];
-              s_f_new[sy] = objective_of(g.sys[sy].op, o);
-            }
-          }
-          if (lane == 0 && !bad) {
-            for (int sy = 0; sy < g.n_sys; ++sy) {
-              FOR_PORTS(p, g.sys[sy].n_o) s_o[sy][p] = s_o_new[sy][p];
-              s_f[sy] = s_f_new[sy];
-            }
-            s_m = m;
-            s_F = combine_of(s_f, g.n_sys, g.combine, g.kind);
-          }
-        }
+        if (badt || m == 0) bad = 1;
+        else if (lane < m) s_px[lane] = px;
+        if (lane == 0) s_m = m;
       }
       if (lane == 0) {
         s_k = k;
@@ -403,6 +476,34 @@ __global__ void __launch_bounds__(kThreads) dbs_tiles_kernel(const __grid_consta
       }
     }
     __syncthreads();
+    if (s_k >= 0 && !s_bad) {
+      if (warp < g.n_sys) {  // one warp per system
+        const int sy = warp;
+        c128 o[kMaxPorts];
+        FOR_PORTS(p, g.sys[sy].n_o) o[p] = s_o[sy][p];
+        const bool ok = accept_pivot_sys(g.sys[sy], lane < s_m ? s_px[lane] : -1, s_m,
+                                         reinterpret_cast<c128*>(gen_smem) + (size_t)sy * kTileMax * kAcceptLd, s_z[sy],
+                                         s_y[sy], s_tz[sy], o);
+        if (lane == 0) {
+          s_sysbad[sy] = !ok;
+          FOR_PORTS(p, g.sys[sy].n_o) s_o_new[sy][p] = o[p];
+          s_f_new[sy] = objective_of(g.sys[sy].op, o);
+        }
+      }
+      __syncthreads();
+      if (tid == 0) {  // committed only if every system's m x m system is regular
+        for (int sy = 0; sy < g.n_sys; ++sy)
+          if (s_sysbad[sy]) s_bad = 1;
+        if (!s_bad) {
+          for (int sy = 0; sy < g.n_sys; ++sy) {
+            FOR_PORTS(p, g.sys[sy].n_o) s_o[sy][p] = s_o_new[sy][p];
+            s_f[sy] = s_f_new[sy];
+          }
+          s_F = combine_of(s_f, g.n_sys, g.combine, g.kind);
+        }
+      }
+      __syncthreads();
+    }
     slot ^= 1;
     ++rd;
     const int k = s_k, pos_k = s_pos;
@@ -461,21 +562,17 @@ __global__ void __launch_bounds__(kThreads) dbs_tiles_kernel(const __grid_consta
     ++n_acc;
     const int m = s_m;
     // U = W[own, K], V = U Z for every system (W, Z read before any update)
-    for (int sy = 0; sy < g.n_sys; ++sy) {
-      const SweepArgs& a = g.sys[sy];
-      c128* U = g.U + (size_t)sy * n * M;
-      c128* V = g.V + (size_t)sy * n * M;
-      for (int q = tid; q < (pe - pb) * m; q += blockDim.x) {
-        const int j = pb + q / m, c = q % m;
-        U[(size_t)j * M + c] = w_sym(a, j, s_px[c]);
-      }
-      __syncthreads();
-      for (int q = tid; q < (pe - pb) * m; q += blockDim.x) {
-        const int j = pb + q / m, c = q % m;
-        c128 acc = mk(0.0, 0.0);
-        for (int b = 0; b < m; ++b) acc = cfma(U[(size_t)j * M + b], s_z[sy][b * kTileMax + c], acc);
-        V[(size_t)j * M + c] = acc;
-      }
+    const int own = pe - pb;
+    for (int q = tid; q < g.n_sys * m * own; q += blockDim.x) {
+      const int sy = q / (m * own), c = q / own % m, j = pb + q % own;
+      g.U[((size_t)sy * M + c) * n + j] = w_sym(g.sys[sy], j, s_px[c]);
+    }
+    __syncthreads();
+    for (int q = tid; q < g.n_sys * m * own; q += blockDim.x) {
+      const int sy = q / (m * own), c = q / own % m, j = pb + q % own;
+      c128 acc = mk(0.0, 0.0);
+      for (int b = 0; b < m; ++b) acc = cfma(g.U[((size_t)sy * M + b) * n + j], s_z[sy][b * kTileMax + c], acc);
+      g.V[((size_t)sy * M + c) * n + j] = acc;
     }
     if (!grid_sync(ctl)) { failed = true; break; }
     // rank-m update of the upper triangle and the state of the own pixels
@@ -483,23 +580,12 @@ __global__ void __launch_bounds__(kThreads) dbs_tiles_kernel(const __grid_consta
       const SweepArgs& a = g.sys[sy];
       const c128* U = g.U + (size_t)sy * n * M;
       const c128* V = g.V + (size_t)sy * n * M;
-      long long e = eb + tid;
-      if (e < ee) {
-        int i, j;
-        tri_rc(e, n, i, j);
-        for (; e < ee; e += blockDim.x) {
-          c128* w = a.W + (size_t)i * a.ldw + j;
-          c128 acc = *w;
-          for (int c = 0; c < m; ++c) acc = cfma(V[(size_t)i * M + c], U[(size_t)j * M + c], acc);
-          *w = acc;
-          tri_step(i, j, n, blockDim.x);
-        }
-      }
+      rank_m_upper(a.W, n, a.ldw, V, U, m, cta, P);
       for (int j = pb + tid; j < pe; j += blockDim.x) {
         c128 dj = a.diag[j], ej = a.e[j];
         for (int c = 0; c < m; ++c) {
-          const c128 u = U[(size_t)j * M + c];
-          dj = cfma(V[(size_t)j * M + c], u, dj);
+          const c128 u = U[(size_t)c * n + j];
+          dj = cfma(V[(size_t)c * n + j], u, dj);
           ej = cfma(u, s_y[sy][c], ej);
         }
         a.diag[j] = dj;
@@ -508,7 +594,7 @@ __global__ void __launch_bounds__(kThreads) dbs_tiles_kernel(const __grid_consta
         for (int p = 0; p < a.n_o; ++p) {
           c128* tp = a.T + (size_t)p * a.ldt + j;
           c128 acc = *tp;
-          for (int c = 0; c < m; ++c) acc = cfma(s_tz[sy][p * kTileMax + c], U[(size_t)j * M + c], acc);
+          for (int c = 0; c < m; ++c) acc = cfma(s_tz[sy][p * kTileMax + c], U[(size_t)c * n + j], acc);
           *tp = acc;
         }
       }
