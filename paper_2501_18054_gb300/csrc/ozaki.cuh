@@ -33,8 +33,9 @@
 // Measured: a tile of K = 64 takes 27,000 cycles of products (544 at 48 cycles:
 // the shared-memory reads of M = 128, N = 64) and 40,000 in all, the rest the
 // read-back (about 120 integer instructions and one FP64 addition per real
-// result).  2048 x 4096 x 64 on 152 SMs: 180 us, 24 TFLOP/s of FP64 products
-// against 1.25 on the FP64 pipe.
+// result).  2048 x 4096 x 64 on 152 SMs: 174 us, 25 TFLOP/s of FP64 products
+// against 1.25 on the FP64 pipe (180 us with a barrier among the read-back
+// warps; accumulators freed in two halves: 184, more spills).
 #pragma once
 
 #include "flush_tc.cuh"
@@ -372,8 +373,8 @@ __device__ __forceinline__ bool oz_tiles(OzState& st, unsigned char* smem, const
   const int tid = threadIdx.x, lane = tid & 31, nwarp = blockDim.x >> 5;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const unsigned s0 = (unsigned)__cvta_generic_to_shared(smem);
-  __shared__ int s_fail, s_efail;
-  if (tid == 0) s_fail = s_efail = 0;
+  __shared__ int s_fail;
+  if (tid == 0) s_fail = 0;
   // earlier generic-proxy use of this shared memory before the bulk copies write it
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
@@ -438,15 +439,13 @@ __device__ __forceinline__ bool oz_tiles(OzState& st, unsigned char* smem, const
       double re[CW];
 #pragma unroll 1
       for (int part = 0; part < 2; ++part) {
-        // one warp waits for the accumulators and the others for it; the
-        // decision to stop is taken by all epilogue threads together
-        if (ew == 0 && !oz_wait_phase(st, OZ_B_FULL)) s_efail = 1;
-        asm volatile("bar.sync 1, %0;" ::"r"(OZ_EW * 32) : "memory");
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        if (s_efail) {
+        // every warp waits for itself (no barrier among them: they drift apart,
+        // and the FP64, integer and memory work of one fills the others' waits)
+        if (!__all_sync(0xffffffffu, oz_wait_phase(st, OZ_B_FULL))) {
           ok = false;
           break;
         }
+        asm volatile("tcgen05.fence::after_thread_sync;");
         // the accumulators are freed once their sums are in registers; all
         // that follows runs beside the products of the next part
         long long V[CW];
