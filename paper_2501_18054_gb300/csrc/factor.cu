@@ -18,13 +18,13 @@
 // cooperative launch does everything: m is known only on the device, and the
 // phases (panel columns above all) are too short for launches of their own.
 //
-// Measured, half the pixels on: N_d = 4096 748 -> 34.5 ms, N_d = 1517 86 -> 9.1
+// Measured, half the pixels on: N_d = 4096 748 -> 32.0 ms, N_d = 1517 86 -> 8.5
 // ms (before: LU of the whole M and its substitutions on the FP64 pipe).  At
-// 4096: panels 10.9 ms (5.3 us a column: one grid barrier, two L2 round trips
-// and the FP64 chain of the reciprocal and the update), products of LU 2.7,
-// of the substitutions 8.0 and of the last step 4.4 (tensor cores and the
-// read-back of ozaki.cuh), diagonal blocks 3.8, interchanges and L^-1 3.0,
-// digits 2.5.
+// 4096: panels 9.6 ms (4.7 us a column: one exchange of words, an L2 round trip
+// for the pivot row and the FP64 chain of the reciprocal and the update; 5.3 us
+// with a grid barrier and a read of the keys), products of LU 2.5, of the
+// substitutions 7.1 and of the last step 4.0 (tensor cores and the read-back of
+// ozaki.cuh), diagonal blocks 3.7, interchanges and L^-1 3.0, digits 2.5.
 #include <cstdio>
 
 #include "factor_common.cuh"
@@ -375,7 +375,7 @@ static FactorScratch factor_scratch(int n, bool images) {
   f.eb = take(images ? ((size_t)n + 1 + OZ_N) * sizeof(int) : 0);
   f.act = take(((size_t)n + 64) * sizeof(int));
   f.cand = take((size_t)2 * 1024 * NB * sizeof(c128));
-  f.key = take((size_t)2 * 1024 * sizeof(unsigned long long));
+  f.key = take((size_t)2 * 1024 * kPanelWord * sizeof(unsigned long long));
   f.cand_row = take((size_t)2 * 1024 * sizeof(int));
   f.drow = take((size_t)2 * NB * sizeof(c128));
   f.piv = take(NB * sizeof(int));
@@ -448,7 +448,9 @@ pngf_status factor_fp64(pngf_ctx* c, const uint8_t* b) {
     return PNGF_ECUDA;
   int P = (n + 15) / 16;
   if (P > c->n_sm) P = c->n_sm;
-  if (cudaMemsetAsync(&a.ctl->bar_count, 0, sizeof(unsigned), s) != cudaSuccess) return PNGF_ECUDA;
+  if (cudaMemsetAsync(&a.ctl->bar_count, 0, sizeof(unsigned), s) != cudaSuccess ||
+      cudaMemsetAsync(a.key, 0, (size_t)2 * P * kPanelWord * sizeof(unsigned long long), s) != cudaSuccess)
+    return PNGF_ECUDA;
   void* params[] = {&a};
   if (cudaLaunchCooperativeKernel((const void*)factor_kernel, dim3(P), dim3(FT_THREADS), params, OZ_SMEM, s) !=
       cudaSuccess)

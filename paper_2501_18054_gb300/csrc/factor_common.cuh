@@ -29,7 +29,7 @@ struct FactorArgs {
   int* ea;
   int* eb;
   c128* cand;               // [2][P][NB] candidate pivot rows
-  unsigned long long* key;  // [2][P] their keys
+  unsigned long long* key;  // [2][P] their keys; factor.cu: words, kPanelWord apart
   int* cand_row;            // [2][P]
   c128* drow;               // [2][NB] diagonal row of the column
   int* piv;                 // NB pivots of the panel
@@ -56,12 +56,15 @@ __device__ __forceinline__ unsigned long long pivot_key(c128 z) {
 // Per column: every CTA publishes its candidate row (and the owner the
 // diagonal row), one grid barrier, every CTA picks the winner, swaps what it
 // owns and updates its rows, tracking the next column's candidate.  The rows
-// travel with the candidates, so one barrier per column is enough.  kDivide: the
-// pivot's reciprocal by FP64 division.
+// travel with the candidates, so one exchange per column is enough: a grid
+// barrier, or (kDivide = false) one word per CTA that every CTA waits for.
+// kDivide: the largest pivot to the last bit and its reciprocal by FP64 division.
+constexpr int kPanelWord = 16;  // 64-bit words between two CTAs' words
 template <int WARPS, bool kDivide>
 __device__ bool factor_panel(const FactorArgs& a, int m, int j0, int jb, c128* ps) {
   __shared__ unsigned long long s_key[WARPS];
-  __shared__ int s_row[WARPS];
+  __shared__ int s_row[WARPS], s_q[WARPS], s_fail;
+  __shared__ unsigned long long s_word;
   __shared__ c128 s_u[NB], s_d[NB];
   __shared__ c128 s_inv;
   __shared__ int s_p;
@@ -69,6 +72,7 @@ __device__ bool factor_panel(const FactorArgs& a, int m, int j0, int jb, c128* p
   const int rows = m - j0;
   const int rb = j0 + (int)((long long)rows * cta / P), re = j0 + (int)((long long)rows * (cta + 1) / P);
   const bool act_lane = lane < jb;
+  if (tid == 0) s_fail = 0;
   unsigned long long bk = 0;
   int br = 0x7fffffff;
   for (int r = rb + warp; r < re; r += WARPS) {
@@ -96,22 +100,76 @@ __device__ bool factor_panel(const FactorArgs& a, int m, int j0, int jb, c128* p
         if (ok > k || (ok == k && orr < r)) { k = ok; r = orr; }
       }
       if (r != 0x7fffffff) a.cand[((size_t)par * P + cta) * NB + lane] = ps[(r - rb) * NB + lane];
-      if (lane == 0) {
+      if (kDivide && lane == 0) {
         a.key[par * P + cta] = k;
         a.cand_row[par * P + cta] = r;
       }
+      if (!kDivide) s_word = r == 0x7fffffff ? 0xffull : (k >> 32 << 32) | (unsigned)(r - rb);
     } else if (warp == 1 && col >= rb && col < re) {
       a.drow[par * NB + lane] = ps[(col - rb) * NB + lane];
     }
-    if (!grid_sync(a.ctl)) return false;
+    if (!kDivide) {
+      // one word per CTA instead of a barrier and a read of the keys: upper half
+      // of the magnitude (a pivot within 2^-20 of the largest), column, row
+      __syncthreads();
+      unsigned long long* words = a.key + (size_t)par * P * kPanelWord;
+      if (tid == 0) {
+        fence_acq_rel_gpu();  // release: the candidate row and the diagonal row
+        *reinterpret_cast<volatile unsigned long long*>(words + (size_t)cta * kPanelWord) =
+            s_word | ((unsigned long long)(unsigned)(col + 1) << 8);
+      }
+      if (tid < ((P + 31) & ~31)) {
+        unsigned k = 0;
+        int r = 0x7fffffff;
+        if (tid < P) {
+          const volatile unsigned long long* w = words + (size_t)tid * kPanelWord;
+          const unsigned long long lim = spin_limit_of(a.ctl), t0 = global_ns();
+          for (unsigned long long it = 0;;) {
+            const unsigned long long v = *w;
+            if (((unsigned)v >> 8) == (unsigned)(col + 1)) {
+              const int local = (int)(v & 0xff);
+              k = (unsigned)(v >> 32);
+              if (local != 0xff) r = j0 + (int)((long long)rows * tid / P) + local;
+              break;
+            }
+            if (++it > lim || ((it & 63) == 0 && global_ns() - t0 > kWaitNs)) {
+              s_fail = 1;
+              latch_status(a.ctl, PNGF_ETIMEOUT);
+              break;
+            }
+          }
+          fence_acq_rel_gpu();  // acquire
+        }
+        const unsigned km = __reduce_max_sync(0xffffffffu, k);
+        const int rm = __reduce_min_sync(0xffffffffu, k == km ? r : 0x7fffffff);
+        const unsigned who = __ballot_sync(0xffffffffu, k == km && r == rm);
+        if (lane == 0) {
+          s_key[warp] = km;
+          s_row[warp] = rm;
+          s_q[warp] = 32 * warp + __ffs(who) - 1;
+        }
+      }
+      __syncthreads();
+      if (s_fail) return false;
+    } else if (!grid_sync(a.ctl)) {
+      return false;
+    }
     // ---- the pivot, its row and its reciprocal (warp 0), the diagonal row (warp 1)
     if (warp == 0) {
       unsigned long long k = 0;
       int r = 0x7fffffff, q = -1;
-      for (int c = lane; c < P; c += 32) {
-        const unsigned long long ck = a.key[par * P + c];
-        const int cr = a.cand_row[par * P + c];
-        if (ck > k || (ck == k && cr < r)) { k = ck; r = cr; q = c; }
+      if (!kDivide) {
+        if (lane < (P + 31) / 32) {
+          k = s_key[lane];
+          r = s_row[lane];
+          q = s_q[lane];
+        }
+      } else {
+        for (int c = lane; c < P; c += 32) {
+          const unsigned long long ck = a.key[par * P + c];
+          const int cr = a.cand_row[par * P + c];
+          if (ck > k || (ck == k && cr < r)) { k = ck; r = cr; q = c; }
+        }
       }
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) {
