@@ -7,7 +7,8 @@
 // design region, possibly of a different size, its own W, state and trace),
 // and one CTA advances one run at a time through the whole search: scoring,
 // selection, the kept-flip update, the FP64 refresh and, on the mixed path,
-// the flush of the delayed set, with only CTA-wide barriers.  All runs of a
+// the flush of the delayed set, with only CTA-wide barriers.  (FP64 batches
+// whose large runs are few go to clusters of four CTAs, batch_cluster.cu.)  All runs of a
 // batch share one stream.  The runs wait in a queue, largest region first, and
 // one CTA per SM takes the next run whenever it finishes one (an atomic
 // counter): a large run then has its SM's FP64 pipe to itself, and the small
@@ -585,6 +586,15 @@ pngf_status run_sweep_batch(pngf_ctx* const* ctxs, int n_runs, int n_sweeps, con
   int grid = c0->n_sm;  // one CTA per SM
   if (grid > n_runs) grid = n_runs;
   if (!mixed && c0->cfg.mode == PNGF_FIRST_IMPROVEMENT) {
+    int max_o = 1, large = 0, min_n = max_n;
+    for (int r = 0; r < n_runs; ++r) {
+      large += 2 * ctxs[r]->cfg.n_d >= max_n;
+      min_n = std::min(min_n, (int)ctxs[r]->cfg.n_d);
+      max_o = std::max(max_o, (int)ctxs[r]->cfg.n_o);
+    }
+    const int clusters = batch_clusters(n_runs, large, min_n, max_n, c0->n_sm);
+    if (clusters > 0)
+      return launch_batch_clusters(ws, n_runs, queue, max_n, max_o, clusters, c0->stream);
     if (cudaFuncSetAttribute(dbs_batch_fp64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM) != cudaSuccess)
       return PNGF_ECUDA;
     dbs_batch_fp64_kernel<<<grid, OZ_THREADS, OZ_SMEM, c0->stream>>>(static_cast<const SweepArgs*>(ws), n_runs, queue);

@@ -56,17 +56,18 @@ struct DelayedArgs {
   int forced_one;           //   or one flip (>= 0)
 };
 
-template <bool kPec>
-__global__ void __launch_bounds__(OZ_THREADS, 1) dbs_delayed_kernel(const __grid_constant__ DelayedArgs g) {
-  const SweepArgs& a = g.a;
-  extern __shared__ __align__(128) unsigned char d_smem[];
-  const int P = gridDim.x, cta = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// CTA `cta` of the P that run one search; the barrier counter and the words of
+// the context are zero when the first of them starts.  Returns false after a
+// timeout.  kBatch: a run of a batch (no active-pixel count, no phase cycles).
+template <bool kPec, bool kBatch>
+__device__ __forceinline__ bool delayed_search(const SweepArgs& a, const int* forced_list, const int* forced_count,
+                                               int forced_one, int P, int cta, unsigned char* d_smem, OzState& oz) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int NW = OZ_THREADS / 32;
   const int n = a.n, n_o = a.n_o;
   const int pb = (int)((long long)n * cta / P), pe = (int)((long long)n * (cta + 1) / P), own = pe - pb;
   Control* ctl = a.ctl;
   const unsigned long long spin_lim = spin_limit_of(ctl);
-  hold_if_asked(ctl);
   const int OSS = own64_stride(n, P), OS = (own + 31) & ~31, nb = OS >> 5;
   c128* s_T = reinterpret_cast<c128*>(d_smem + OZ_SMEM);  // [n_o][OSS]
   c128* s_diag = s_T + n_o * OSS;
@@ -81,8 +82,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_delayed_kernel(const __grid
   c128* const Xn = s_ac + OSS;                           // [kDelay64][OS]
   const bool x_near = (size_t)(kChains64 + 3 + kDelay64) * OSS * sizeof(c128) <= (size_t)OZ_SMEM;
   const bool best_mode = kPec && a.mode == PNGF_BEST_IMPROVEMENT;
-  const bool forced = kPec && (g.forced != nullptr || g.forced_one >= 0);
-  const int n_forced = !forced ? 0 : g.forced ? *g.forced_count : 1;
+  const bool forced = kPec && (forced_list != nullptr || forced_one >= 0);
+  const int n_forced = !forced ? 0 : forced_list ? *forced_count : 1;
   const size_t ldx = a.ldt;
   __shared__ int s_pos[kOwn64];
   __shared__ unsigned char s_b[kOwn64];
@@ -95,8 +96,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_delayed_kernel(const __grid
   __shared__ int s_best[2];                  // earliest improving position of the own pixels, by round parity
   __shared__ unsigned s_key[2];              // smallest key of the round
   __shared__ int s_fail;
-  __shared__ __align__(8) unsigned long long s_bars[OZ_NBAR];
-  __shared__ unsigned s_tmem;
+  __syncthreads();  // every thread is done with an earlier search's arrays
   if (tid == 0) {
     s_op = a.op;
     FOR_PORTS(p, n_o) s_o[p] = ctl->o[p];
@@ -130,11 +130,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_delayed_kernel(const __grid
     if (!a.order) s_pos[jl] = j;
   }
   load_state();
-  OzState oz;
-  oz_setup(oz, s_bars, &s_tmem);
   long long n_acc = 0, n_evals = 0, n_refresh = 0, sum_active = 0;
   int sweeps_done = 0, converged = 0, status = PNGF_OK;
-  const bool timer = cta == 0 && tid == 0;
+  const bool timer = !kBatch && cta == 0 && tid == 0;
   __shared__ long long ph[16];  // phase cycles, kept by the timer thread only
   if (timer)
     for (int q = 0; q < 16; ++q) ph[q] = 0;
@@ -158,7 +156,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_delayed_kernel(const __grid
       if ((unsigned)px < (unsigned)n) a.pos_of[px] = q;
       else latch_status(ctl, PNGF_EINVAL);
     }
-    if (!grid_sync(ctl)) return false;
+    if (!grid_sync(ctl, P)) return false;
     if (*reinterpret_cast<volatile int*>(&ctl->status) == PNGF_EINVAL) status = PNGF_EINVAL;
     for (int jl = tid; jl < own; jl += blockDim.x) s_pos[jl] = a.pos_of[pb + jl];
     __syncthreads();
@@ -167,14 +165,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_delayed_kernel(const __grid
   // folds the delayed set into W
   auto fold = [&]() -> bool {
     if (r == 0) return true;
-    if (!grid_sync(ctl)) return false;  // every CTA's part of the columns
+    if (!grid_sync(ctl, P)) return false;  // every CTA's part of the columns
     fold64_digits(a.X64, ldx, s_al, a.last64, r, n, a.ozA, a.ozB, a.ozEa, a.ozEb, cta * NW + warp, P * NW);
     fold64_bases(a.W, a.ldw, a.X64, ldx, s_invd, s_hist, a.last64, kPec ? a.b : nullptr, r, n, cta * (int)blockDim.x + tid, P * (int)blockDim.x);
-    if (!grid_sync(ctl)) return false;
+    if (!grid_sync(ctl, P)) return false;
     const bool ok = fold64_product(oz, d_smem, a.W, a.ldw, n, r, a.ozA, a.ozB, a.ozEa, a.ozEb, cta, P);
     if (!ok && tid == 0) latch_status(ctl, PNGF_ETIMEOUT);
     r = 0;
-    if (!ok || !grid_sync(ctl)) return false;
+    if (!ok || !grid_sync(ctl, P)) return false;
     for (int jl = tid; jl < own; jl += blockDim.x) {
       s_last[jl] = -1;
       a.last64[pb + jl] = -1;
@@ -197,7 +195,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_delayed_kernel(const __grid
     double fn = 0.0;
     c128 al = mk(0.0, 0.0), co = al, idv = al;
     int pos = INT_MAX;
-    const int k_forced = !forced ? -1 : n_acc >= n_forced ? -1 : g.forced ? g.forced[n_acc] : g.forced_one;
+    const int k_forced = !forced ? -1 : n_acc >= n_forced ? -1 : forced_list ? forced_list[n_acc] : forced_one;
     if (forced && (k_forced < 0 || k_forced >= n)) break;  // all done (the list holds pixels of the region)
     bool ok = false;
     if (tid < own) {
@@ -445,20 +443,22 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_delayed_kernel(const __grid
       store_state(false);
       __syncthreads();
       refresh_x(a, pb, pe);
-      if (!grid_sync(ctl)) { failed = true; break; }
+      if (!grid_sync(ctl, P)) { failed = true; break; }
       tick(8);
       const int m_act = refresh_residual(a, pb, pe, act);
       sum_active += m_act;
+      if (cta == 0)  // for the correction, after the next barrier
+        for (int q = tid; q < m_act; q += blockDim.x) a.actg[q] = act[q];
       const int t_end = count_below(act, m_act, pe - 1);
-      if (!grid_sync(ctl)) { failed = true; break; }
+      if (!grid_sync(ctl, P)) { failed = true; break; }
       tick(9);
       correct_strips<false>(a, pb, pe, a.actg, t_end, reinterpret_cast<float*>(d_smem), OZ_SMEM);
-      if (!grid_sync(ctl)) { failed = true; break; }
+      if (!grid_sync(ctl, P)) { failed = true; break; }
       tick(10);
-      ports_partial(a, pb, pe);
-      if (!grid_sync(ctl)) { failed = true; break; }
+      ports_partial(a, pb, pe, cta);
+      if (!grid_sync(ctl, P)) { failed = true; break; }
       load_state();
-      ports_total(a, s_o);
+      ports_total(a, s_o, P);
       if (tid == 0) s_f = objective_of(s_op, s_o);
       __syncthreads();
       tick(11);
@@ -477,21 +477,33 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_delayed_kernel(const __grid
   if (!failed && !fold()) failed = true;  // what a break left in the set
   __syncthreads();
   store_state(true);
-  oz_teardown(oz, failed);
   if (cta == 0 && tid == 0) {
     if (failed) status = PNGF_ETIMEOUT;
     FOR_PORTS(p, n_o) ctl->o[p] = s_o[p];
     ctl->f = s_f;
     if (!kPec) ctl->since_refresh = since_refresh;
     if (!forced) ctl->n_acc_total += (int)n_acc;
-    const long long cnt[8] = {n_acc, n_evals, sweeps_done, converged, n_refresh, 0, status, sum_active};
-    ph[7] = clock64() - t_begin;
+    const long long cnt[8] = {n_acc, n_evals, sweeps_done, converged, n_refresh, 0, status, kBatch ? 0 : sum_active};
+    if (timer) ph[7] = clock64() - t_begin;
     for (int q = 0; q < 8 && !forced; ++q) ctl->counters[q] = cnt[q];
-    for (int q = 0; q < 16; ++q) ctl->phase_cycles[q] = ph[q];
+    for (int q = 0; q < 16 && !kBatch; ++q) ctl->phase_cycles[q] = ph[q];
     if (a.counters && !forced)
       for (int q = 0; q < 8; ++q) a.counters[q] = cnt[q];
     if (status != PNGF_OK && status != PNGF_ECAPACITY) latch_status(ctl, status);
   }
+  return !failed;
+}
+
+template <bool kPec>
+__global__ void __launch_bounds__(OZ_THREADS, 1) dbs_delayed_kernel(const __grid_constant__ DelayedArgs g) {
+  extern __shared__ __align__(128) unsigned char d_smem[];
+  __shared__ __align__(8) unsigned long long s_bars[OZ_NBAR];
+  __shared__ unsigned s_tmem;
+  hold_if_asked(g.a.ctl);
+  OzState oz;
+  oz_setup(oz, s_bars, &s_tmem);
+  const bool ok = delayed_search<kPec, false>(g.a, g.forced, g.forced_count, g.forced_one, gridDim.x, blockIdx.x, d_smem, oz);
+  oz_teardown(oz, !ok);
 }
 
 // CTAs of the delayed search, or 0 where it does not apply (FP64: BEST mode,

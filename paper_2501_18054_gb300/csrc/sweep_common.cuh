@@ -109,14 +109,13 @@ __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_re
 // old / P, which is complete once the counter reaches (old / P + 1) P.  One
 // atomic per CTA and no generation word, so the last arrival releases the
 // others without a further round trip.  The spin is bounded: on expiry the
-// CTA latches PNGF_ETIMEOUT and returns false.
-__device__ bool grid_sync(Control* ctl) {
+// CTA latches PNGF_ETIMEOUT and returns false.  P: the CTAs that meet.
+__device__ bool grid_sync(Control* ctl, unsigned P) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
     fence_acq_rel_gpu();  // release: this CTA's writes before its arrival
-    const unsigned P = gridDim.x;
     const unsigned long long lim = spin_limit_of(ctl);
     const unsigned old = atomicAdd(&ctl->bar_count, 1u);
     const unsigned target = (old / P + 1) * P;
@@ -136,6 +135,8 @@ __device__ bool grid_sync(Control* ctl) {
   __syncthreads();
   return s_ok != 0;
 }
+
+__device__ __forceinline__ bool grid_sync(Control* ctl) { return grid_sync(ctl, gridDim.x); }
 
 // Test hook of the timeout path (pngf_set_wait_limit): CTA hold_cta - 1 waits
 // on a flag that nothing sets, bounded by a longer wait than the others' own
@@ -841,7 +842,7 @@ __device__ void correct_strips(const SweepArgs& a, int pb, int pe, const int* ac
 }
 
 // partial o sums of pixels [pb, pe) -> opart[cta]
-__device__ __noinline__ void ports_partial(const SweepArgs& a, int pb, int pe) {
+__device__ __noinline__ void ports_partial(const SweepArgs& a, int pb, int pe, int cta) {
   __shared__ c128 red[kMaxPorts][kMaxWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int p = 0; p < a.n_o; ++p) {
@@ -858,19 +859,20 @@ __device__ __noinline__ void ports_partial(const SweepArgs& a, int pb, int pe) {
   if (threadIdx.x < a.n_o) {
     c128 s = mk(0.0, 0.0);
     for (int q = 0; q < (int)(blockDim.x >> 5); ++q) s = cadd(s, red[threadIdx.x][q]);
-    a.opart[(size_t)blockIdx.x * a.n_o + threadIdx.x] = s;
+    a.opart[(size_t)cta * a.n_o + threadIdx.x] = s;
   }
 }
+__device__ __forceinline__ void ports_partial(const SweepArgs& a, int pb, int pe) { ports_partial(a, pb, pe, blockIdx.x); }
 
 // o_p = c_o,p + sum over the CTAs of their partial sums (after a grid
 // barrier): warp p adds port p's partials in a fixed lane order and tree, so
 // every CTA obtains the same value; the FP64 adds run on one warp per port.
-__device__ void ports_total(const SweepArgs& a, c128* o_out) {
+__device__ void ports_total(const SweepArgs& a, c128* o_out, int P) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (warp < a.n_o) {
     const int p = warp;
     c128 acc = mk(0.0, 0.0);
-    for (int q = lane; q < (int)gridDim.x; q += 32) acc = cadd(acc, a.opart[(size_t)q * a.n_o + p]);
+    for (int q = lane; q < P; q += 32) acc = cadd(acc, a.opart[(size_t)q * a.n_o + p]);
     for (int off = 16; off > 0; off >>= 1) {
       acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
       acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
@@ -879,6 +881,8 @@ __device__ void ports_total(const SweepArgs& a, c128* o_out) {
   }
   __syncthreads();
 }
+
+__device__ __forceinline__ void ports_total(const SweepArgs& a, c128* o_out) { ports_total(a, o_out, gridDim.x); }
 
 SweepArgs make_args(pngf_ctx* c) {
   SweepArgs a{};
