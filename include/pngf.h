@@ -398,6 +398,8 @@ pngf_status pngf_restore(pngf_ctx* ctx);
  * delayed set (mixed), [4] state update (and the rank-1 update of W on the
  * FP64 path), [5] refreshes, [6] sweep set-up, [7] whole kernel,
  * [8..11] refresh sub-phases (x, residual, correction, ports), [12..15] 0.
+ * FP64 FIRST and PEC searches: [2] fetch of the winner, [3] the column, [4]
+ * state update, [5] 0, [12] folds of the delayed set.
  * Synchronizes the stream.
  */
 pngf_status pngf_get_phase_cycles(pngf_ctx* ctx, int64_t* host16);

@@ -1,7 +1,7 @@
 // Kept-flip update of the FP64 maintained inverse, W += alpha c c^T (Eq. 9 in
 // field form; complex symmetric W, upper triangle), with the scaled column
-// ac = alpha c formed once per kept flip.  Used by the persistent FP64 search
-// and the batch kernel; one complex FMA per element of the triangle.
+// ac = alpha c formed once per kept flip.  Used by the rank-1 FP64
+// search and the batch kernel's BEST mode; one complex FMA per element of the triangle.
 #pragma once
 
 #include "sweep_common.cuh"

@@ -1,4 +1,7 @@
-// Direct binary search on the device (FP64 path).
+// Direct binary search on the device (FP64 path).  FIRST mode runs on the
+// delayed-update kernel of delayed_search.cuh; the rank-1 kernel below serves BEST
+// mode and contexts whose CTAs hold more pixels than that kernel takes.  Both
+// follow the same steps; single kept flips (pngf_accept_flip) are at the end.
 //
 // Per kept flip of pixel k (section "Low-rank update evaluation", Eqs. 9-14 in
 // the field form of Supplementary Note 4; the cost split of Supplementary
@@ -14,7 +17,7 @@
 //           of e and T against G (residuals r = c_d - M e, R = G_od - T M^T,
 //           corrections (I + W V) r and R (I + V W)), then o = c_o + G_od V e
 //
-// One cooperative launch runs the whole search.  Pixels are split into
+// One cooperative launch runs the whole search.  In the rank-1 kernel pixels are split into
 // contiguous chunks, one per CTA; the packed upper triangle of W is split
 // into equal element ranges, one per CTA.  Grid-wide barriers are a counter
 // plus generation word with a bounded spin: a barrier that waits longer than
