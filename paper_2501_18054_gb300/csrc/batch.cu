@@ -414,6 +414,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_batch_fp64_kernel(const Swe
         break;
       }
       if (best == INT_MAX) {
+        __syncthreads();  // every thread has read s_best and s_bad: the next chunk's scoring writes them
         n_evals += chunk_end - t;
         t = chunk_end;
         if (t < n) continue;

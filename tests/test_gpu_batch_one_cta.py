@@ -1,0 +1,62 @@
+"""FP64 batches with one CTA per run: regions of more than one scoring chunk (128
+positions), folds of more than one row block (128 rows) inside a sweep, the
+refresh of a whole run by one CTA, and regions above 1024 pixels.
+
+A run of fewer than four pixels, or one above 1024, keeps the whole batch on one
+CTA per run.  Every run is compared with the same run done alone, bit for bit
+without refreshes (the same arithmetic) and to 1e-12 with them (the ports and
+corrections of a refresh are summed in another order: 2**-53 times the terms'
+number), and its final state with a solve of its final design (1e-12, the bound
+of test_gpu_delayed.py for the same systems).  Many chunks hold no improving flip
+(late sweeps), many sweeps end with an empty delayed set.
+"""
+import numpy as np
+import pytest
+
+from paper_2501_18054_gb300 import workloads as W
+from test_gpu_delayed import _case, _solve
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    from paper_2501_18054_gb300 import build as B
+    B.build()
+    from paper_2501_18054_gb300 import pngf
+    return pngf
+
+
+@pytest.mark.parametrize("refresh_k", [0, 64])
+@pytest.mark.parametrize("sizes", [(130, 3, 300, 257, 128), (1030, 129)])
+def test_one_cta_batch_equals_solo(P, sizes, refresh_k):
+    sweeps = 6
+    runs = []
+    for i, n in enumerate(sizes):
+        runs.append((_case(n, 13 * n + i, 1 + i % 3), W.random_design(n, i), W.shuffled_order(n, sweeps, seed=i) if i % 2 == 0 else None))
+
+    def context(case, b):
+        c = P.DbsContext(case, tau=1e-9, refresh_k=refresh_k)
+        c.factor(b)
+        return c
+
+    ctxs = [context(case, b) for case, b, _ in runs]
+    res = P.DbsBatch(ctxs).dbs_sweep(sweeps, orders=[o for _, _, o in runs])
+    for c, r, (case, b, order) in zip(ctxs, res, runs):
+        s = context(case, b)
+        rs = s.dbs_sweep(sweeps, order=order)
+        assert np.array_equal(r["trace"], rs["trace"]) and np.array_equal(c.design(), s.design())
+        assert np.array_equal(r["counters"][:7], rs["counters"][:7])
+        if case.n_d > 256:
+            assert np.bincount(r["trace"][:, 0]).max() > 64  # folds inside a sweep
+        a, e = c.state(with_W=True), s.state(with_W=True)
+        Wm, ex, T, o = _solve(case, c.design())
+        iu = np.triu_indices(case.n_d)
+        for x, y, z in [(a["diag"], e["diag"], np.diag(Wm)), (a["e"], e["e"], ex), (a["T"], e["T"], T),
+                        (a["W"][iu], e["W"][iu], Wm[iu]), (c.eval_ports()[0], s.eval_ports()[0], o)]:
+            bar = 1e-12 * np.max(np.abs(z))
+            assert np.max(np.abs(x - z)) <= bar
+            assert np.array_equal(x, y) if refresh_k == 0 else np.max(np.abs(x - y)) <= bar
+        s.close()
+    for c in ctxs:
+        c.close()
