@@ -195,6 +195,7 @@ __device__ __forceinline__ bool delayed_search(const SweepArgs& a, const int* fo
     double fn = 0.0;
     c128 al = mk(0.0, 0.0), co = al, idv = al;
     int pos = INT_MAX;
+    const double f_round = kPec ? s_f : 0.0;  // BEST mode decides by it after warp 0 may have moved on to the new s_f
     const int k_forced = !forced ? -1 : n_acc >= n_forced ? -1 : forced_list ? forced_list[n_acc] : forced_one;
     if (forced && (k_forced < 0 || k_forced >= n)) break;  // all done (the list holds pixels of the region)
     bool ok = false;
@@ -293,9 +294,8 @@ __device__ __forceinline__ bool delayed_search(const SweepArgs& a, const int* fo
         gb = rec_at(tid)->gain;
       }
       block_best(gb, pix);
-      const double f = s_f;
-      key = pix != INT_MAX && improves64(s_op, rec_at((int)(((long long)(pix + 1) * P - 1) / n))->f_new, f,
-                                         accept_threshold(s_op, f))
+      key = pix != INT_MAX && improves64(s_op, rec_at((int)(((long long)(pix + 1) * P - 1) / n))->f_new, f_round,
+                                         accept_threshold(s_op, f_round))
                 ? (unsigned)pix
                 : kNoKey64;
     }
