@@ -342,14 +342,6 @@ __device__ __forceinline__ void oz_ld_groups(unsigned addr, float d[4 * OZ_G]) {
   for (int q = 0; q < 32; ++q) d[q] = __uint_as_float(u[q]);
 }
 
-// 32 bytes (two entries of C) per access
-__device__ __forceinline__ void oz_ld2(const c128* p, c128& a, c128& b) {
-  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a.x), "=d"(a.y), "=d"(b.x), "=d"(b.y) : "l"(p) : "memory");
-}
-__device__ __forceinline__ void oz_st2(c128* p, c128 a, c128 b) {
-  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(a.x), "d"(a.y), "d"(b.x), "d"(b.y) : "memory");
-}
-
 // The tiles [t_begin, T) with step t_step, in a pipeline of three roles:
 //   lane 0 of warp 1 streams the operand chunks through two buffers.  The
 //   chunks 0 .. nk-1 are needed for the real part and again for the imaginary
@@ -361,7 +353,7 @@ __device__ __forceinline__ void oz_st2(c128* p, c128 a, c128 b) {
 //   with it C += A B^T (OP = +1), C -= A B^T (-1) or C = A B^T (0).
 //   tile_of(t, I, J)      tile t: A row block I, B row block J
 //   row_of(r, J, cols)    C at the first column of tile column J for row r of
-//                         A (32-byte aligned; nullptr: no such row), and how
+//                         A (nullptr: no such row), and how
 //                         many of the tile's columns exist
 // smem: OZ_SMEM bytes, 128-byte aligned; the CTA has at least OZ_THREADS
 // threads.  Returns false after a timeout (the caller then calls
@@ -468,11 +460,8 @@ __device__ __forceinline__ bool oz_tiles(OzState& st, unsigned char* smem, const
           if (left <= 0) continue;
           c128 x[4];
           if (OP != 0 && part == 1) {
-            x[1] = x[2] = x[3] = mk(0.0, 0.0);
-            if (left >= 2) oz_ld2(p, x[0], x[1]);
-            else x[0] = p[0];
-            if (left >= 4) oz_ld2(p + 2, x[2], x[3]);
-            else if (left == 3) x[2] = p[2];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = u < left ? p[u] : mk(0.0, 0.0);
           }
           const int4 e4 = ebp[q];
           const int e_b[4] = {e4.x, e4.y, e4.z, e4.w};
@@ -490,10 +479,11 @@ __device__ __forceinline__ bool oz_tiles(OzState& st, unsigned char* smem, const
             else if (OP > 0) x[u] = mk(x[u].x + re[4 * q + u], x[u].y + v[u]);
             else x[u] = mk(x[u].x - re[4 * q + u], x[u].y - v[u]);
           }
-          if (left >= 2) oz_st2(p, x[0], x[1]);
-          else p[0] = x[0];
-          if (left >= 4) oz_st2(p + 2, x[2], x[3]);
-          else if (left == 3) p[2] = x[2];
+          // 16 bytes per access: with a 256-bit store in its place (st.global.v4.f64)
+          // nvcc 13.0.88 left the store out, in code that two kernels of a file call
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (u < left) p[u] = x[u];
         }
       }
     }

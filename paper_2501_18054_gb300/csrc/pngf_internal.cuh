@@ -166,10 +166,6 @@ __host__ __forceinline__ T* at(pngf_ctx* c, size_t off) {
 // factor.cu
 pngf_status factor_fp64(pngf_ctx* c, const uint8_t* b);
 pngf_status factor_mixed(pngf_ctx* c, const uint8_t* b);
-// batch_cluster.cu: FP64 batches on clusters of CTAs (runs: the device's argument table)
-int batch_clusters(int n_runs, int large, int min_n, int max_n, int n_sm);
-pngf_status launch_batch_clusters(const void* runs, int n_runs, int* queue, int max_n, int max_o, int clusters,
-                                  cudaStream_t stream);
 size_t factor_scratch_bytes(int n, bool images);
 void factor_images(int n, size_t off[5]);  // offsets of the digit images A, B and the row exponents in the scratch, and their end
 // sweep_mixed.cu

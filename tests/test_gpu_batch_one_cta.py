@@ -1,4 +1,4 @@
-"""FP64 batches with one CTA per run: regions of more than one scoring chunk (128
+"""FP64 batches, above all with one CTA per run: regions of more than one scoring chunk (128
 positions), folds of more than one row block (128 rows) inside a sweep, the
 refresh of a whole run by one CTA, and regions above 1024 pixels.
 
@@ -59,4 +59,21 @@ def test_one_cta_batch_equals_solo(P, sizes, refresh_k):
             assert np.array_equal(x, y) if refresh_k == 0 else np.max(np.abs(x - y)) <= bar
         s.close()
     for c in ctxs:
+        c.close()
+
+
+@pytest.mark.parametrize("sizes", [(600, 257, 300)])
+def test_cluster_batch_of_larger_regions(P, sizes):
+    """Few large runs, on clusters: shares of more than 64 pixels, whose delayed
+    columns are read from global memory; W against a solve."""
+    ctxs, cases = [], [_case(n, 5 * n + i, 1 + i) for i, n in enumerate(sizes)]
+    for i, case in enumerate(cases):
+        ctxs.append(P.DbsContext(case, tau=1e-9, refresh_k=50))
+        ctxs[-1].factor(W.random_design(case.n_d, i))
+    for c, case, r in zip(ctxs, cases, P.DbsBatch(ctxs).dbs_sweep(4)):
+        assert len(r["trace"]) > 64
+        Wm, e, T, o = _solve(case, c.design())
+        st, iu = c.state(with_W=True), np.triu_indices(case.n_d)
+        for x, z in [(st["diag"], np.diag(Wm)), (st["e"], e), (st["T"], T), (st["W"][iu], Wm[iu]), (c.eval_ports()[0], o)]:
+            assert np.max(np.abs(x - z)) <= 1e-12 * np.max(np.abs(z))
         c.close()
