@@ -69,15 +69,7 @@ Layout make_layout(const pngf_config& cfg) {
   L.xs = take(mixed ? (1 + n_o) * n * 8 * sizeof(float) : 0);
   L.xadd = take(mixed ? (size_t)L.R * 4 * sizeof(float) : 0);  // alpha_i of the mixed search as double-words
   const bool fp64 = cfg.precision == PNGF_FP64;
-  size_t im[5];
-  factor_images(cfg.n_d, im);
-  L.oz = take(pec ? im[4] : factor_scratch_bytes(cfg.n_d, fp64));
-  if (!mixed) {
-    L.ozA = L.oz + im[0];
-    L.ozB = L.oz + im[1];
-    L.ozEa = L.oz + im[2];
-    L.ozEb = L.oz + im[3];
-  }
+  L.oz = take(pec ? oz_operand_bytes(cfg.n_d) : factor_scratch_bytes(cfg.n_d, fp64));
   L.X64 = take(mixed ? 0 : (size_t)kDelay64 * L.ldt * c);
   L.last64 = take(mixed ? 0 : n * sizeof(int));
   L.snapW = take(L.snapW_bytes);

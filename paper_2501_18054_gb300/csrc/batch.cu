@@ -376,10 +376,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_batch_fp64_kernel(const Swe
     auto fold = [&]() -> bool {
       if (r == 0) return true;
       __syncthreads();
-      fold64_digits(a.X64, ldx, s_al, a.last64, r, n, a.ozA, a.ozB, a.ozEa, a.ozEb, warp, NW);
+      fold64_digits(a.X64, ldx, s_al, a.last64, r, n, a.oz, warp, NW);
       fold64_bases(a.W, a.ldw, a.X64, ldx, s_invd, s_hist, a.last64, nullptr, r, n, tid, blockDim.x);
       __syncthreads();
-      const bool ok = fold64_product(oz, b_smem, a.W, a.ldw, n, r, a.ozA, a.ozB, a.ozEa, a.ozEb, 0, 1);
+      const bool ok = fold64_product(oz, b_smem, a.W, a.ldw, n, r, a.oz, 0, 1);
+      if (const unsigned m = ok ? oz_listed(a.oz) : 0u) {
+        fold64_redo(a.W, a.ldw, n, r, a.oz, m, warp, NW);
+        __syncthreads();
+      }
       for (int q = tid; q < n; q += blockDim.x) {
         a.last64[q] = -1;
         a.diag[q] = a.W[(size_t)q * a.ldw + q];  // d is formed from the matrix's own diagonal
@@ -609,7 +613,7 @@ static int batch_clusters(int n_runs, int large, int min_n, int max_n, int n_sm)
 }
 
 static pngf_status launch_batch_clusters(const void* runs, int n_runs, int* queue, int max_n, int max_o, int clusters,
-                                  cudaStream_t stream) {
+                                         cudaStream_t stream) {
   if (cudaFuncSetAttribute(dbs_batch_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)kDelayed64MaxSmem) != cudaSuccess)
     return PNGF_ECUDA;

@@ -123,12 +123,12 @@ __device__ __forceinline__ c128 delayed_entry(c128 base, const c128* s, int ld) 
 // ---------------------------------------------------------------- fold
 // Operand images of the fold: A rows y_j = alpha 2^-h x_j, B rows 2^h x_j, where
 // 2^h is about |alpha|^(1/2): both sides then carry the square root of their
-// column's contribution to W, and the fixed point of a row, relative to its
-// largest entry, resolves every contribution relative to the largest one.
+// column's contribution to W, and the fixed point of a row is relative to its
+// largest contribution.
 // X[i ldx + j]: column i at pixel j; s_al: alpha_i; entries up to a pixel's last
 // flip are zero.  Warps gw of nw.
 __device__ __noinline__ void fold64_digits(const c128* X, size_t ldx, const c128* s_al, const int* last, int r, int n,
-                                           unsigned char* imgA, unsigned char* imgB, int* ea, int* eb, int gw, int nw) {
+                                           const OzOperands& im, int gw, int nw) {
   const int nk = (r + OZ_KC - 1) / OZ_KC, qa = (n + OZ_M - 1) / OZ_M * (OZ_M / 4), qb = (n + OZ_N - 1) / OZ_N * (OZ_N / 4);
   auto half_scale = [&](int k) {  // the double 2^h
     const c128 al = s_al[k];
@@ -137,20 +137,21 @@ __device__ __noinline__ void fold64_digits(const c128* X, size_t ldx, const c128
   };
   for (int q = gw; q < qa + qb; q += nw) {
     if (q < qa)
-      oz_digitise_rows<OZ_M>(4 * q, r, nk, imgA, ea, [&](int j, int k) {
+      oz_digitise_rows<OZ_M>(4 * q, r, nk, im.A, im.sqA, im.ea, im.na, im.fa, [&](int j, int k) {
         if (j >= n || k <= last[j]) return mk(0.0, 0.0);
         const double s = half_scale(k), is = __longlong_as_double((2046ll << 52) - __double_as_longlong(s));  // 1 / s
         const c128 al = s_al[k];
         return cmul(mk(al.x * is, al.y * is), X[(size_t)k * ldx + j]);
       });
     else
-      oz_digitise_rows<OZ_N>(4 * (q - qa), r, nk, imgB, eb, [&](int j, int k) {
+      oz_digitise_rows<OZ_N>(4 * (q - qa), r, nk, im.B, im.sqB, im.eb, im.nb, im.fb, [&](int j, int k) {
         if (j >= n || k <= last[j]) return mk(0.0, 0.0);
         const double s = half_scale(k);
         const c128 x = X[(size_t)k * ldx + j];
         return mk(x.x * s, x.y * s);
       });
   }
+  if (gw == 0 && (threadIdx.x & 31) == 0) oz_list_clear(im);
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
@@ -174,12 +175,15 @@ __device__ __forceinline__ int fold64_tiles(int n) {
   const int nI = (n + OZ_M - 1) / OZ_M, nJ = (n + OZ_N - 1) / OZ_N;
   return nI * nJ - nI * (nI - 1);
 }
+__device__ __forceinline__ c128* fold64_row(c128* W, int ldw, int n, int j, int J, int& cols) {
+  cols = n - J * OZ_N;
+  return j < n ? W + (size_t)j * ldw + J * OZ_N : nullptr;
+}
 __device__ __noinline__ bool fold64_product(OzState& oz, unsigned char* smem, c128* W, int ldw, int n, int r,
-                                            const unsigned char* imgA, const unsigned char* imgB, const int* ea,
-                                            const int* eb, int t_begin, int t_step) {
+                                            const OzOperands& im, int t_begin, int t_step) {
   const int nI = (n + OZ_M - 1) / OZ_M, nJ = (n + OZ_N - 1) / OZ_N;
   return oz_tiles<1>(
-      oz, smem, imgA, imgB, ea, eb, (r + OZ_KC - 1) / OZ_KC, fold64_tiles(n), t_begin, t_step,
+      oz, smem, im, r, (float)r, fold64_tiles(n), t_begin, t_step,
       [&](long long t, int& I, int& J) {  // row block I starts at tile I nJ - I (I - 1)
         int lo = 0, hi = nI - 1;
         while (lo < hi) {
@@ -190,10 +194,11 @@ __device__ __noinline__ bool fold64_product(OzState& oz, unsigned char* smem, c1
         I = lo;
         J = 2 * lo + (int)t - (lo * nJ - lo * (lo - 1));
       },
-      [&](int j, int J, int& cols) -> c128* {
-        cols = n - J * OZ_N;
-        return j < n ? W + (size_t)j * ldw + J * OZ_N : nullptr;
-      });
+      [&](int j, int J, int& cols) { return fold64_row(W, ldw, n, j, J, cols); });
+}
+// the m entries that the product left to FP64 (after a barrier), warps gw of nw
+__device__ __noinline__ void fold64_redo(c128* W, int ldw, int n, int r, const OzOperands& im, unsigned m, int gw, int nw) {
+  oz_redo<1>(im, m, r, gw, nw, [&](int j, int J, int& cols) { return fold64_row(W, ldw, n, j, J, cols); });
 }
 
 }  // namespace

@@ -166,13 +166,17 @@ __device__ __forceinline__ bool delayed_search(const SweepArgs& a, const int* fo
   auto fold = [&]() -> bool {
     if (r == 0) return true;
     if (!grid_sync(ctl, P)) return false;  // every CTA's part of the columns
-    fold64_digits(a.X64, ldx, s_al, a.last64, r, n, a.ozA, a.ozB, a.ozEa, a.ozEb, cta * NW + warp, P * NW);
+    fold64_digits(a.X64, ldx, s_al, a.last64, r, n, a.oz, cta * NW + warp, P * NW);
     fold64_bases(a.W, a.ldw, a.X64, ldx, s_invd, s_hist, a.last64, kPec ? a.b : nullptr, r, n, cta * (int)blockDim.x + tid, P * (int)blockDim.x);
     if (!grid_sync(ctl, P)) return false;
-    const bool ok = fold64_product(oz, d_smem, a.W, a.ldw, n, r, a.ozA, a.ozB, a.ozEa, a.ozEb, cta, P);
+    const bool ok = fold64_product(oz, d_smem, a.W, a.ldw, n, r, a.oz, cta, P);
     if (!ok && tid == 0) latch_status(ctl, PNGF_ETIMEOUT);
-    r = 0;
     if (!ok || !grid_sync(ctl, P)) return false;
+    if (const unsigned m = oz_listed(a.oz)) {
+      fold64_redo(a.W, a.ldw, n, r, a.oz, m, warp * P + cta, P * NW);
+      if (!grid_sync(ctl, P)) return false;
+    }
+    r = 0;
     for (int jl = tid; jl < own; jl += blockDim.x) {
       s_last[jl] = -1;
       a.last64[pb + jl] = -1;

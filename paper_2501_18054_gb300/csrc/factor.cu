@@ -18,13 +18,13 @@
 // cooperative launch does everything: m is known only on the device, and the
 // phases (panel columns above all) are too short for launches of their own.
 //
-// Measured, half the pixels on: N_d = 4096 748 -> 32.0 ms, N_d = 1517 86 -> 8.5
+// Measured, half the pixels on: N_d = 4096 748 -> 38 ms, N_d = 1517 86 -> 9.5
 // ms (before: LU of the whole M and its substitutions on the FP64 pipe).  At
-// 4096: panels 9.6 ms (4.7 us a column: one exchange of words, an L2 round trip
+// 4096 the panels take 9.6 ms (4.7 us a column: one exchange of words, an L2 round trip
 // for the pivot row and the FP64 chain of the reciprocal and the update; 5.3 us
-// with a grid barrier and a read of the keys), products of LU 2.5, of the
-// substitutions 7.1 and of the last step 4.0 (tensor cores and the read-back of
-// ozaki.cuh), diagonal blocks 3.7, interchanges and L^-1 3.0, digits 2.5.
+// with a grid barrier and a read of the keys), the products of LU, substitutions and
+// last step about 17 (tensor cores and the read-back of
+// ozaki.cuh), diagonal blocks 3.7, interchanges and L^-1 3.0, digits 4.
 #include <cstdio>
 
 #include "factor_common.cuh"
@@ -130,6 +130,17 @@ __global__ void contrast_kernel(const c128* G, const c128* dv, const uint8_t* b,
   if (threadIdx.x == 0) *high = h;
 }
 
+// After a product: the grid's barrier, and the entries that the product left to FP64
+template <int OP, class Row>
+__device__ __forceinline__ bool product_done(const FactorArgs& a, bool ok, int K, Row row_of) {
+  if (!ok || !grid_sync(a.ctl)) return false;
+  const unsigned m = oz_listed(a.im);
+  if (m == 0) return true;
+  const int P = gridDim.x;
+  oz_redo<OP>(a.im, m, K, (int)(threadIdx.x >> 5) * P + blockIdx.x, P * FT_WARPS, row_of);
+  return grid_sync(a.ctl);
+}
+
 // ---------------------------------------------------------------- the factorisation
 __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_constant__ FactorArgs a) {
   extern __shared__ __align__(128) unsigned char f_smem[];
@@ -138,7 +149,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
   __shared__ unsigned s_tmem;
   __shared__ Swaps s_sw;
   __shared__ int s_cum[264];  // tiles before row block I of the last product (n_d <= 32768: 257 blocks)
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, P = gridDim.x, cta = blockIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, P = gridDim.x, cta = blockIdx.x;
   const int gw = cta * FT_WARPS + warp, nw = P * FT_WARPS;  // warps of the grid
   const int n = a.n, ldw = a.ldw, ncol = n + 1;
   Control* ctl = a.ctl;
@@ -175,17 +186,19 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
   auto digits_rhs = [&](int i0, int K) {
     const int nk = (K + OZ_KC - 1) / OZ_KC;
     for (int r0 = 4 * gw; r0 < nJ * OZ_N; r0 += 4 * nw)
-      oz_digitise_rows<OZ_N>(r0, K, nk, a.imgB, a.eb, [&](int c, int k) {
+      oz_digitise_rows<OZ_N>(r0, K, nk, a.im.B, a.im.sqB, a.im.eb, a.im.nb, a.im.fb, [&](int c, int k) {
         return c < ncol ? a.W[(size_t)act[i0 + k] * ldw + c] : mk(0.0, 0.0);
       });
   };
   auto digits_A = [&](int rows, int K, auto load) {
     const int nk = (K + OZ_KC - 1) / OZ_KC, rpad = (rows + OZ_M - 1) / OZ_M * OZ_M;
     for (int r0 = 4 * gw; r0 < rpad; r0 += 4 * nw)
-      oz_digitise_rows<OZ_M>(r0, K, nk, a.imgA, a.ea, [&](int r, int k) { return r < rows ? load(r, k) : mk(0.0, 0.0); });
+      oz_digitise_rows<OZ_M>(r0, K, nk, a.im.A, a.im.sqA, a.im.ea, a.im.na, a.im.fa,
+                             [&](int r, int k) { return r < rows ? load(r, k) : mk(0.0, 0.0); });
   };
   // the images are read next by bulk asynchronous copies (async proxy)
   auto images_done = [&]() -> bool {
+    if (cta == 0 && tid == 0) oz_list_clear(a.im);
     asm volatile("fence.proxy.async.global;" ::: "memory");
     return grid_sync(ctl);
   };
@@ -221,17 +234,17 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
     // U12, column by column
     const int nI = (rest + OZ_M - 1) / OZ_M, nb1 = (rest + OZ_N - 1) / OZ_N;
     for (int r0 = 4 * gw; r0 < nb1 * OZ_N; r0 += 4 * nw)
-      oz_digitise_rows<OZ_N>(r0, jb, nk, a.imgB, a.eb, [&](int r, int k) {
+      oz_digitise_rows<OZ_N>(r0, jb, nk, a.im.B, a.im.sqB, a.im.eb, a.im.nb, a.im.fb, [&](int r, int k) {
         return r < rest ? a.LU[(size_t)(j0 + k) * ldw + i1 + r] : mk(0.0, 0.0);
       });
     if (!(ok = images_done())) break;
-    ok = oz_tiles<-1>(oz, f_smem, a.imgA, a.imgB, a.ea, a.eb, nk, (long long)nI * nb1, cta, P,
-                      [&](long long t, int& I, int& J) { I = (int)(t % nI); J = (int)(t / nI); },
-                      [&](int r, int J, int& cols) -> c128* {
-                        cols = rest - J * OZ_N;
-                        return r < rest ? a.LU + (size_t)(i1 + r) * ldw + i1 + J * OZ_N : nullptr;
-                      });
-    if (ok) ok = grid_sync(ctl);
+    auto row = [&](int r, int J, int& cols) -> c128* {
+      cols = rest - J * OZ_N;
+      return r < rest ? a.LU + (size_t)(i1 + r) * ldw + i1 + J * OZ_N : nullptr;
+    };
+    ok = oz_tiles<-1>(oz, f_smem, a.im, jb, 1.0f, (long long)nI * nb1, cta, P,
+                      [&](long long t, int& I, int& J) { I = (int)(t % nI); J = (int)(t / nI); }, row);
+    ok = product_done<-1>(a, ok, jb, row);
   }
   // ---- the pivoted right-hand sides, and the inverses of the diagonal blocks
   //      of L and U, by which the substitutions become products
@@ -251,30 +264,31 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
   //      X_b = (diagonal block)^-1 Y_b, then Y -= (rest of the block column) X_b
   for (int step = 0; ok && step < 2 * nblk; ++step) {
     const bool fwd = step < nblk;
-    const int bi = fwd ? step : 2 * nblk - 1 - step, i0 = bi * BB, jb = min(BB, m - i0), nk = (jb + OZ_KC - 1) / OZ_KC;
+    const int bi = fwd ? step : 2 * nblk - 1 - step, i0 = bi * BB, jb = min(BB, m - i0);
     const c128* inv = a.binv + ((size_t)(fwd ? 0 : nblk) + bi) * BB * BB;
     digits_rhs(i0, jb);
     digits_A(jb, jb, [&](int r, int k) { return inv[r * BB + k]; });
     if (!(ok = images_done())) break;
-    ok = oz_tiles<0>(oz, f_smem, a.imgA, a.imgB, a.ea, a.eb, nk, nJ, cta, P,
-                     [&](long long t, int& I, int& J) { I = 0; J = (int)t; },
-                     [&](int r, int J, int& cols) -> c128* {
-                       cols = ncol - J * OZ_N;
-                       return r < jb ? a.W + (size_t)act[i0 + r] * ldw + J * OZ_N : nullptr;
-                     });
-    if (!ok || !(ok = grid_sync(ctl))) break;
+    auto block_row = [&](int r, int J, int& cols) -> c128* {
+      cols = ncol - J * OZ_N;
+      return r < jb ? a.W + (size_t)act[i0 + r] * ldw + J * OZ_N : nullptr;
+    };
+    ok = oz_tiles<0>(oz, f_smem, a.im, jb, 0.0f, nJ, cta, P, [&](long long t, int& I, int& J) { I = 0; J = (int)t; },
+                     block_row);
+    ok = product_done<0>(a, ok, jb, block_row);
+    if (!ok) break;
     const int r0 = fwd ? i0 + jb : 0, rows = fwd ? m - r0 : i0, nI = (rows + OZ_M - 1) / OZ_M;
     if (rows == 0) continue;
     digits_rhs(i0, jb);
     digits_A(rows, jb, [&](int r, int k) { return a.LU[(size_t)(r0 + r) * ldw + i0 + k]; });
     if (!(ok = images_done())) break;
-    ok = oz_tiles<-1>(oz, f_smem, a.imgA, a.imgB, a.ea, a.eb, nk, (long long)nI * nJ, cta, P,
-                      [&](long long t, int& I, int& J) { I = (int)(t % nI); J = (int)(t / nI); },
-                      [&](int r, int J, int& cols) -> c128* {
-                        cols = ncol - J * OZ_N;
-                        return r < rows ? a.W + (size_t)act[r0 + r] * ldw + J * OZ_N : nullptr;
-                      });
-    if (ok) ok = grid_sync(ctl);
+    auto row = [&](int r, int J, int& cols) -> c128* {
+      cols = ncol - J * OZ_N;
+      return r < rows ? a.W + (size_t)act[r0 + r] * ldw + J * OZ_N : nullptr;
+    };
+    ok = oz_tiles<-1>(oz, f_smem, a.im, jb, 1.0f, (long long)nI * nJ, cta, P,
+                      [&](long long t, int& I, int& J) { I = (int)(t % nI); J = (int)(t / nI); }, row);
+    ok = product_done<-1>(a, ok, jb, row);
   }
   // ---- the rows of the pixels that are off, and T: += G_ia v_a [W | e]_a, of W
   //      only the tiles that reach the upper triangle
@@ -292,14 +306,23 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
     __syncthreads();
     const int T = s_cum[nI];
     for (int k0 = 0; ok && k0 < m; k0 += OZ_KMAX) {
-      const int kb = min(OZ_KMAX, m - k0), nk = (kb + OZ_KC - 1) / OZ_KC;
+      const int kb = min(OZ_KMAX, m - k0);
       digits_rhs(k0, kb);
       digits_A(nr, kb, [&](int r, int k) {
         const int pk = act[k0 + k];
         return cmul(r < ni ? a.G[(size_t)ina[r] * n + pk] : a.God[(size_t)(r - ni) * n + pk], a.dv[pk]);
       });
       if (!(ok = images_done())) break;
-      ok = oz_tiles<1>(oz, f_smem, a.imgA, a.imgB, a.ea, a.eb, nk, T, cta, P,
+      auto row = [&](int r, int J, int& cols) -> c128* {
+        if (r >= nr) return nullptr;
+        if (r < ni) {
+          cols = ncol - J * OZ_N;
+          return a.W + (size_t)ina[r] * ldw + J * OZ_N;
+        }
+        cols = n - J * OZ_N;
+        return a.T + (size_t)(r - ni) * a.ldt + J * OZ_N;
+      };
+      ok = oz_tiles<1>(oz, f_smem, a.im, kb, 1.0f, T, cta, P,
                        [&](long long t, int& I, int& J) {
                          int lo = 0, hi = nI - 1;
                          while (lo < hi) {
@@ -310,16 +333,8 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
                          I = lo;
                          J = jmin(I) + (int)t - s_cum[I];
                        },
-                       [&](int r, int J, int& cols) -> c128* {
-                         if (r >= nr) return nullptr;
-                         if (r < ni) {
-                           cols = ncol - J * OZ_N;
-                           return a.W + (size_t)ina[r] * ldw + J * OZ_N;
-                         }
-                         cols = n - J * OZ_N;
-                         return a.T + (size_t)(r - ni) * a.ldt + J * OZ_N;
-                       });
-      if (ok) ok = grid_sync(ctl);
+                       row);
+      ok = product_done<1>(a, ok, kb, row);
     }
   }
   // ---- the lower triangle of W mirrors the upper one; diag W and e are read off
@@ -356,23 +371,52 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
 
 }  // namespace
 
-// the factor's scratch (c->L.oz): digit images (not for mixed contexts), row
-// exponents, lists, candidate rows, reciprocals of the pivots
+// operands of up to n + kMaxPorts rows (A) and n + 1 rows (B), K <= OZ_KMAX; rows in
+// whole blocks
+static size_t oz_operands_at(char* p, int n, OzOperands& im) {
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    char* q = p + off;
+    off += (bytes + 255) / 256 * 256;
+    return q;
+  };
+  const size_t ra = (size_t)n + kMaxPorts + OZ_M, rb = (size_t)n + 1 + OZ_N;
+  im.A = reinterpret_cast<unsigned char*>(take(oz_a_bytes(n + kMaxPorts, OZ_KMAX)));
+  im.B = reinterpret_cast<unsigned char*>(take(oz_b_bytes(n + 1, OZ_KMAX)));
+  im.sqA = reinterpret_cast<unsigned char*>(take(oz_a_bytes(n + kMaxPorts, OZ_KMAX) / (2 * OZ_S)));
+  im.sqB = reinterpret_cast<unsigned char*>(take(oz_b_bytes(n + 1, OZ_KMAX) / (2 * OZ_S)));
+  im.ea = reinterpret_cast<int*>(take(ra * sizeof(int)));
+  im.eb = reinterpret_cast<int*>(take(rb * sizeof(int)));
+  im.na = reinterpret_cast<float*>(take(ra * sizeof(float)));
+  im.nb = reinterpret_cast<float*>(take(rb * sizeof(float)));
+  im.fa = reinterpret_cast<c128*>(take(ra * OZ_KMAX * sizeof(c128)));
+  im.fb = reinterpret_cast<c128*>(take(rb * OZ_KMAX * sizeof(c128)));
+  im.list = reinterpret_cast<unsigned*>(take((1 + ((size_t)n + kMaxPorts) * (n + 1)) * sizeof(unsigned)));
+  return off;
+}
+OzOperands oz_operands(char* scratch, int n) {
+  OzOperands im;
+  oz_operands_at(scratch, n, im);
+  return im;
+}
+size_t oz_operand_bytes(int n) {
+  OzOperands im;
+  return oz_operands_at(nullptr, n, im);
+}
+
+// the factor's scratch (c->L.oz): operand images (not for mixed contexts), lists,
+// candidate rows, reciprocals of the pivots
 struct FactorScratch {
-  size_t imgA, imgB, ea, eb, act, cand, key, cand_row, drow, piv, dinv, perm, binv, high, total;
+  size_t act, cand, key, cand_row, drow, piv, dinv, perm, binv, high, total;
 };
 static FactorScratch factor_scratch(int n, bool images) {
   FactorScratch f{};
-  size_t off = 0;
+  size_t off = images ? oz_operand_bytes(n) : 0;
   auto take = [&](size_t bytes) {
     const size_t o = off;
     off += (bytes + 255) / 256 * 256;
     return o;
   };
-  f.imgA = take(images ? oz_a_bytes(n + kMaxPorts, OZ_KMAX) : 0);
-  f.imgB = take(images ? oz_b_bytes(n + 1, OZ_KMAX) : 0);
-  f.ea = take(images ? ((size_t)n + kMaxPorts + OZ_M) * sizeof(int) : 0);
-  f.eb = take(images ? ((size_t)n + 1 + OZ_N) * sizeof(int) : 0);
   f.act = take(((size_t)n + 64) * sizeof(int));
   f.cand = take((size_t)2 * 1024 * NB * sizeof(c128));
   f.key = take((size_t)2 * 1024 * kPanelWord * sizeof(unsigned long long));
@@ -387,14 +431,6 @@ static FactorScratch factor_scratch(int n, bool images) {
   return f;
 }
 size_t factor_scratch_bytes(int n, bool images) { return factor_scratch(n, images).total; }
-void factor_images(int n, size_t off[5]) {
-  const FactorScratch f = factor_scratch(n, true);
-  off[0] = f.imgA;
-  off[1] = f.imgB;
-  off[2] = f.ea;
-  off[3] = f.eb;
-  off[4] = f.act;  // the end of the four
-}
 
 // ---------------------------------------------------------------- driver
 // arguments of both factorisations
@@ -420,10 +456,7 @@ FactorArgs factor_args(pngf_ctx* c, const uint8_t* b) {
   a.diag = at<c128>(c, c->L.diag);
   a.e = at<c128>(c, c->L.e);
   a.Gs = at<double>(c, c->L.gsum);
-  a.imgA = reinterpret_cast<unsigned char*>(ws + f.imgA);
-  a.imgB = reinterpret_cast<unsigned char*>(ws + f.imgB);
-  a.ea = reinterpret_cast<int*>(ws + f.ea);
-  a.eb = reinterpret_cast<int*>(ws + f.eb);
+  if (c->cfg.precision == PNGF_FP64) a.im = oz_operands(ws, n);
   a.act = reinterpret_cast<int*>(ws + f.act);
   a.count = a.act + n + 32;
   a.cand = reinterpret_cast<c128*>(ws + f.cand);

@@ -24,10 +24,7 @@ struct FactorArgs {
   int* act;    // the m pixels that are on, ascending, then the n - m others
   int* count;  // m
   const int* high;  // device: whether the contrast is high (contrast_kernel)
-  unsigned char* imgA;
-  unsigned char* imgB;
-  int* ea;
-  int* eb;
+  OzOperands im;
   c128* cand;               // [2][P][NB] candidate pivot rows
   unsigned long long* key;  // [2][P] their keys; factor.cu: words, kPanelWord apart
   int* cand_row;            // [2][P]

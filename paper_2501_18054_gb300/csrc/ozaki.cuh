@@ -5,17 +5,27 @@
 //   C[i][j] +-= sum_{k<K} A[i][k] B[j][k],   K <= 64, everything complex128
 //
 // Every row of A and of B is scaled by a power of two (its own largest real or
-// imaginary part lies below 2^e) and written in fixed point, X = rint(a 2^(54-e)),
-// |X| <= 2^54: 7 signed base-256 digits, each a whole number in [-128, 127]
-// that bf16 holds exactly.  A product of two digits is below 2^14 and the
+// imaginary part lies below 2^e) and written in fixed point, X = rint(a 2^(55-e)):
+// 7 signed base-256 digits, each a whole number in [-128, 127]
+// that bf16 holds exactly.  A product of two digits is at most 2^14 and the
 // sums of one accumulator (all digit pairs s + t = g of a K of 64, two
 // products per complex part) stay below 2^24, so that the FP32 accumulation of
 // tcgen05.mma is exact whole-number arithmetic: the order of the additions
 // does not matter and the result is the same for every tile shape and grid.
-// The pairs with s + t <= 7 are kept (34 of 49); the rest are below
-// 2^-58 of the largest product.  The dominant error is the rounding of the
-// operands to 55 bits of their row's largest entry, below the 53-bit rounding
-// of an FP64 multiply-add chain of the same length.
+// The pairs with s + t <= 7 are kept (34 of 49); the rest are 2^-60 of the product
+// of the scales.
+//
+// Accuracy, against a chain of FP64 multiply-adds: what is lost is the rounding of
+// the operands to 56 bits of their row's largest entry, 2^-56 of the product
+// 2^(ea + eb) of the two rows' scales, where a chain loses some 2^-52 of the sum's
+// size.  Where a row of A and a row of B are large at the same k the digits win.
+// Where they are large at different k
+// (two parts of a region that hardly couple, metal between two pixels) every
+// term is small against the scales and the digits would keep fewer bits.  So
+//   m2 = sum_k |A_ik|^2 |B_jk|^2   (relative to the scales)
+// is formed first, by one more bf16 product of squared magnitudes, and the
+// entries where the digits' error exceeds a chain's (oz_lossy) are listed and
+// summed in FP64 from the operands themselves (oz_redo), by every warp of the grid.
 //
 // Why: the FP64 pipe of this part issues 1.7 multiply-adds per clock and SM
 // (1.25 TFLOP/s in all).  136 bf16 products replace the four FP64 products of
@@ -31,11 +41,14 @@
 // N = 256 (measured): 64 columns per part cost half of 32 columns of both.
 //
 // Measured: a tile of K = 64 takes 27,000 cycles of products (544 at 48 cycles:
-// the shared-memory reads of M = 128, N = 64) and 40,000 in all, the rest the
-// read-back (about 120 integer instructions and one FP64 addition per real
-// result).  2048 x 4096 x 64 on 152 SMs: 174 us, 25 TFLOP/s of FP64 products
-// against 1.25 on the FP64 pipe (180 us with a barrier among the read-back
-// warps; accumulators freed in two halves: 184, more spills).
+// the shared-memory reads of M = 128, N = 64) and 49,000 in all, bound by the
+// issue of the read-back (about 120 integer instructions and one FP64 addition per
+// real result; 96 registers a thread, some of them spilled).  2048 x 4096 x 64 on
+// 152 SMs: 217 us, 20 TFLOP/s of FP64 products against 1.25 on the FP64 pipe.
+// (With no sums in FP64 and C in 256-bit accesses 174 us; see there.)  Entries
+// summed in FP64, 64 flips at N_d = 1024 of lossy metal: a fifth of the triangle,
+// 0.07 ms on 64 CTAs; in a dielectric guide 10^-4 of the substitutions' diagonal
+// blocks and none elsewhere.
 #pragma once
 
 #include "flush_tc.cuh"
@@ -58,7 +71,7 @@ constexpr int OZ_NBUF = 2;
 constexpr int OZ_SMEM = OZ_NBUF * OZ_BUF;     // 168 KB: one CTA per SM
 constexpr int OZ_TMEM = OZ_G * OZ_N;          // all 512 columns
 constexpr int OZ_EW = 16;                     // epilogue warps (the last ones of the CTA)
-constexpr int OZ_THREADS = 32 * (2 + OZ_EW);  // 112 registers a thread
+constexpr int OZ_THREADS = 32 * (2 + OZ_EW);
 constexpr int kOzNaN = 0x20000000;            // row exponent of a row with an infinity or NaN
 
 static_assert(OZ_TMEM == 512, "tensor memory");
@@ -76,13 +89,18 @@ __host__ __device__ __forceinline__ size_t oz_b_bytes(int rows, int K) {
 }
 
 // ---------------------------------------------------------------- digits
-// X = rint(x 2^(54 - e)), e = emax - 1022 (biased exponent emax of the row's
-// largest entry), plus the offset that turns its base-256 digits into bytes:
+// Biased exponent of the scale of a row whose largest entry has the upper word
+// hmax (without its sign): one more than the entry's where X with the digits'
+// offsets would not fit 56 bits (from 127.498 / 128 of a power of two on: the
+// mantissa's upper bits 0xFDFE0; 0xFDF00 is taken).
+__device__ __forceinline__ int oz_scale_exp(int hmax) { return (hmax + 0x2100) >> 20; }
+// X = rint(x 2^(55 - e)), e = emax - 1022 (emax: oz_scale_exp of the row), plus the
+// offset that turns its base-256 digits into bytes:
 // byte 6 - s of the result is digit s + 128.  Integer arithmetic only.
 __device__ __forceinline__ unsigned long long oz_fixed(double x, int emax) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
   const int E = (int)(u >> 52) & 0x7ff;
-  unsigned long long m = E ? ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 1 : 0ull;
+  unsigned long long m = E ? ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 2 : 0ull;
   const int d = emax - E;
   if (d > 0) m = d < 60 ? (m + (1ull << (d - 1))) >> d : 0ull;
   const unsigned long long X = (long long)u < 0 ? 0ull - m : m;
@@ -126,32 +144,83 @@ __device__ __forceinline__ void oz_store_digits(unsigned char* base, int sub, co
   oz_store8<6>(base, sub, y);
 }
 
+// x 2^-e as a float (20 bits), e = emax - 1022; integer arithmetic only
+__device__ __forceinline__ float oz_scaled(double x, int emax) {
+  const int hi = __double2hiint(x), d = ((hi >> 20) & 0x7ff) - emax;
+  return d < -100 ? 0.0f : __int_as_float(((126 + d) << 23) | ((hi & 0xfffff) << 3));
+}
+
 // One warp digitises four rows of an operand with nk chunks (K <= 64): lane =
 // (row << 3) | group of 8 k.  `load(row, k)` returns the entry (zero past the
-// operand's edges).  BLK = rows per image block (128: A, 64: B).
+// operand's edges).  BLK = rows per image block (128: A, 64: B).  sq: the squared
+// magnitudes in bf16; entries below 2^-30 of the row's largest count as 2^-60, so
+// that a sum of them is zero only where every product is.  norms: their sum over the
+// row; infinity for a row that holds an infinity or NaN.  full: the entries
+// themselves.
 template <int BLK, class Load>
-__device__ __forceinline__ void oz_digitise_rows(int row0, int K, int nk, unsigned char* img, int* exps, Load load) {
+__device__ __forceinline__ void oz_digitise_rows(int row0, int K, int nk, unsigned char* img, unsigned char* sq, int* exps,
+                                                 float* norms, c128* full, Load load) {
   constexpr int SUB = BLK * OZ_KC * 2;
   const int lane = threadIdx.x & 31, row = row0 + (lane >> 3), kg = lane & 7;
   double re[8], im[8];
-  int emax = 0;
+  int hmax = 0;
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const int k = kg * 8 + u;
     const c128 z = k < K ? load(row, k) : mk(0.0, 0.0);
     re[u] = z.x;
     im[u] = z.y;
-    emax = max(emax, max(oz_exp(z.x), oz_exp(z.y)));
+    hmax = max(hmax, max(__double2hiint(z.x) & 0x7fffffff, __double2hiint(z.y) & 0x7fffffff));
   }
 #pragma unroll
-  for (int off = 1; off < 8; off <<= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, off));
-  if (kg == 0) exps[row] = emax == 0x7ff ? kOzNaN : emax - 1022;
+  for (int off = 1; off < 8; off <<= 1) hmax = max(hmax, __shfl_xor_sync(0xffffffffu, hmax, off));
+  const int emax = oz_scale_exp(hmax);
+  float q[8], norm = 0.0f;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const float x = oz_scaled(re[u], emax), y = oz_scaled(im[u], emax);
+    q[u] = (oz_exp(re[u]) | oz_exp(im[u])) && emax < 0x7ff ? fmaxf(fmaf(x, x, y * y), 0x1p-60f) : 0.0f;
+    norm += q[u];
+  }
+#pragma unroll
+  for (int off = 1; off < 8; off <<= 1) norm += __shfl_xor_sync(0xffffffffu, norm, off);
+  if (kg == 0) {
+    exps[row] = emax >= 0x7ff ? kOzNaN : emax - 1022;
+    norms[row] = emax >= 0x7ff ? INFINITY : norm;
+  }
   if (kg < 2 * nk) {
-    unsigned char* base = img + ((size_t)(row / BLK) * nk + (kg >> 1)) * (2 * OZ_S * SUB) +
-                          oz_off(row % BLK, (kg & 1) * 8);
+    const size_t chunk = (size_t)(row / BLK) * nk + (kg >> 1);
+    const int at = oz_off(row % BLK, (kg & 1) * 8);
+    unsigned char* base = img + chunk * (2 * OZ_S * SUB) + at;
     oz_store_digits(base, SUB, re, emax);
     oz_store_digits(base + OZ_S * SUB, SUB, im, emax);
+    uint4 v;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(v.x) : "f"(q[1]), "f"(q[0]));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(v.y) : "f"(q[3]), "f"(q[2]));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(v.z) : "f"(q[5]), "f"(q[4]));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(v.w) : "f"(q[7]), "f"(q[6]));
+    *reinterpret_cast<uint4*>(sq + chunk * SUB + at) = v;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) full[(size_t)row * OZ_KMAX + kg * 8 + u] = mk(re[u], im[u]);
   }
+}
+
+// Whether an entry is less accurate by its digits than as an FP64 chain, in rms
+// errors of a real part, in units of 2^(ea + eb - 53):
+//   digits: operands rounded to 2^-56 of their scales, and the sum to 2^-55 of
+//           their product, (na + nb + 1) / 192;
+//   chain:  a rounding of 2^-53 0.41 of the partial sum per step, sums growing to
+//           (m2 / 2)^(1/2) like a random walk: 0.168 K m2 / 2.
+// na, nb: norms of the two rows.
+__device__ __forceinline__ bool oz_lossy(float na, float nb, float m2, float K) {
+  const float s = na + nb + 1.0f;
+  return s > 16.1f * K * m2 && (m2 > 0.0f || s == INFINITY);
+}
+// Whether the rounding of C itself (`roundings` of them in the chain: one where a
+// sum is added at the end, K where every term is added to C) exceeds that error all
+// the same: 0.168 roundings |C|^2; emax: biased exponent of C's larger part
+__device__ __forceinline__ bool oz_below_c(float na, float nb, float roundings, int emax, int e_ab) {
+  return na + nb + 1.0f < 32.2f * roundings * exp2f(2.0f * (float)(emax - 1023 - e_ab));
 }
 
 // ---------------------------------------------------------------- tile products
@@ -245,17 +314,28 @@ __device__ __forceinline__ void oz_teardown(OzState& st, bool failed) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(st.tmem), "r"(OZ_TMEM));
 }
 
-__device__ __forceinline__ void oz_issue_copy(const OzState& st, int bf, unsigned sbuf, const unsigned char* a,
-                                              const unsigned char* b) {
-  const unsigned mb = st.mb0 + 8 * (OZ_B_LOAD + bf);
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(OZ_BUF) : "memory");
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(sbuf),
-               "l"(a), "r"(OZ_ACHUNK), "r"(mb)
+// one copy's barrier, and its pieces
+__device__ __forceinline__ void oz_expect(const OzState& st, int bf, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(st.mb0 + 8 * (OZ_B_LOAD + bf)), "r"(bytes)
                : "memory");
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   sbuf + OZ_ACHUNK),
-               "l"(b), "r"(OZ_BCHUNK), "r"(mb)
+}
+__device__ __forceinline__ void oz_copy(const OzState& st, int bf, unsigned dst, const unsigned char* src, unsigned bytes) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(st.mb0 + 8 * (OZ_B_LOAD + bf))
                : "memory");
+}
+
+// The squared magnitudes of OZ_SQ tiles at a time, OZ_SQ / 2 in a buffer: one
+// accumulator each.  (One tile at a time, the products of the next tile's real
+// part wait until the read-back warps are through with the tile before.)
+constexpr int OZ_SQ = 6;
+constexpr int OZ_SQ_A = OZ_KMAX / OZ_KC * OZ_ASUB, OZ_SQ_TILE = OZ_SQ_A + OZ_KMAX / OZ_KC * OZ_BSUB;
+static_assert(OZ_SQ / OZ_NBUF * OZ_SQ_TILE <= OZ_BUF && OZ_SQ * OZ_N <= OZ_TMEM, "squares of a group of tiles");
+__device__ __forceinline__ void oz_issue_squares(const OzState& st, unsigned tile_buf, int acc, int nk) {
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  for (int c = 0; c < nk; ++c)
+    oz_mma(st.tmem + (unsigned)acc * OZ_N, oz_desc(tile_buf + c * OZ_ASUB), oz_desc(tile_buf + OZ_SQ_A + c * OZ_BSUB),
+           oz_idesc(false), c > 0 ? 1u : 0u);
 }
 
 // the 68 products of one chunk for one part of the tile (0: re, 1: im):
@@ -283,11 +363,11 @@ __device__ __forceinline__ void oz_issue_mma(const OzState& st, unsigned sbuf, i
   }
 }
 
-// The digit groups' whole-number sums D_0 .. D_7 -> sum_g D_g 256^(7 - g) 2^-13
-// (the product X Y in units of 2^53), rounded; below 2^62 in magnitude.  The
-// sums up to D_2 are below 2^22 and turn into integers by an addition of
+// The digit groups' whole-number sums D_0 .. D_7 -> sum_g D_g 256^(7 - g) 2^-15
+// (the product X Y in units of 2^55), rounded; below 2^62 in magnitude.  The
+// sums D_0 and D_1 are at most 2^22 and turn into integers by an addition of
 // 1.5 2^23; D_6 and D_7 matter to a part of their range only and are joined in
-// FP32 (their rounding there is below 2^-5 units).
+// FP32 (their rounding there is below 2^-7 units).
 __device__ __forceinline__ long long oz_mad(int a, int b, long long c) {
   long long r;
   asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
@@ -297,12 +377,12 @@ __device__ __forceinline__ long long oz_fixed_sum(const float* d, int stride) {
   constexpr float kMagic = 12582912.0f;  // 1.5 2^23
   constexpr int kBits = 0x4B400000;
   const int D0 = __float_as_int(d[0] + kMagic) - kBits, D1 = __float_as_int(d[stride] + kMagic) - kBits;
-  const int D2 = __float_as_int(d[2 * stride] + kMagic) - kBits;
+  const int D2 = __float2int_rn(d[2 * stride]);
   const int D3 = __float2int_rn(d[3 * stride]), D4 = __float2int_rn(d[4 * stride]), D5 = __float2int_rn(d[5 * stride]);
-  const float low = fmaf(d[7 * stride], 0.00390625f, d[6 * stride]);        // D_6 + D_7 / 256
-  const int t = __float_as_int(fmaf(low, 0.03125f, kMagic)) - kBits;        // / 32, rounded
+  const float low = fmaf(d[7 * stride], 0.00390625f, d[6 * stride]);  // D_6 + D_7 / 256
+  const int t = __float_as_int(fmaf(low, 0.0078125f, kMagic)) - kBits;  // / 128, rounded
   const long long H = oz_mad(D0, 1 << 24, oz_mad(D1, 1 << 16, oz_mad(D2, 256, (long long)D3)));
-  return (H << 19) + oz_mad(D4, 2048, oz_mad(D5, 8, (long long)t));
+  return (H << 17) + oz_mad(D4, 512, oz_mad(D5, 2, (long long)t));
 }
 
 // V 2^sh rounded to FP64 (NaN past its range).  Integer arithmetic only: an FP64 instruction
@@ -342,26 +422,93 @@ __device__ __forceinline__ void oz_ld_groups(unsigned addr, float d[4 * OZ_G]) {
   for (int q = 0; q < 32; ++q) d[q] = __uint_as_float(u[q]);
 }
 
+// 16 consecutive columns of one accumulator for this thread's lane
+__device__ __forceinline__ void oz_ld_squares(unsigned addr, float d[16]) {
+  unsigned u[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
+        "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
+      : "r"(addr));
+#pragma unroll
+  for (int q = 0; q < 16; ++q) d[q] = __uint_as_float(u[q]);
+}
+
+// The list of the entries to sum again: (row of A << 16) | row of B.  oz_listed: how
+// many, after a barrier that follows the product; oz_list_clear: by one thread
+// before the barrier ahead of it.
+__device__ __forceinline__ unsigned oz_listed(const OzOperands& im) { return *reinterpret_cast<volatile unsigned*>(im.list); }
+__device__ __forceinline__ void oz_list_clear(const OzOperands& im) { *im.list = 0; }
+
+// marks: bit u = column j0 + u of this lane's row r
+__device__ __forceinline__ void oz_list_add(const OzOperands& im, unsigned marks, int r, int j0) {
+  const int lane = threadIdx.x & 31, cnt = __popc(marks);
+  int incl = cnt;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += y;
+  }
+  unsigned at = 0;
+  if (lane == 31) at = atomicAdd(im.list, (unsigned)incl);
+  at = __shfl_sync(0xffffffffu, at, 31) + (unsigned)(incl - cnt);
+  for (; marks; marks &= marks - 1) im.list[1 + at++] = (unsigned)r << 16 | (unsigned)(j0 + __ffs(marks) - 1);
+}
+
+// Sums the m listed entries in FP64: four lanes an entry, lane q of them the terms k
+// = q, q + 4, ..., their sums added pairwise.  Warps gw of nw.  Bound by the FP64 pipe
+// (four instructions of 64 cycles for eight terms).
+template <int OP, class Row>
+__device__ __forceinline__ void oz_redo(const OzOperands& im, unsigned m, int K, int gw, int nw, Row row_of) {
+  const int lane = threadIdx.x & 31, part = lane & 3;
+  for (unsigned e0 = 8u * gw; e0 < m; e0 += 8u * nw) {
+    const unsigned e = e0 + (lane >> 2);
+    const unsigned at = e < m ? im.list[1 + e] : 0u;
+    const int r = (int)(at >> 16), j = (int)(at & 0xffffu);
+    const c128* fa = im.fa + (size_t)r * OZ_KMAX;
+    const c128* fb = im.fb + (size_t)j * OZ_KMAX;
+    c128 s = mk(0.0, 0.0);
+    if (e < m) {
+#pragma unroll 8
+      for (int k = part; k < K; k += 4) s = cfma(fa[k], fb[k], s);
+    }
+#pragma unroll
+    for (int off = 1; off < 4; off <<= 1) {
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+    }
+    if (e < m && part == 0) {
+      int cols;
+      c128* p = row_of(r, j / OZ_N, cols) + j % OZ_N;
+      *p = OP == 0 ? s : OP > 0 ? cadd(*p, s) : csub(*p, s);
+    }
+  }
+}
+
 // The tiles [t_begin, T) with step t_step, in a pipeline of three roles:
-//   lane 0 of warp 1 streams the operand chunks through two buffers.  The
-//   chunks 0 .. nk-1 are needed for the real part and again for the imaginary
-//   part, which starts with the two chunks still in the buffers;
+//   lane 0 of warp 1 streams the operands through two buffers: before every
+//   OZ_SQ-th tile the squared magnitudes of the next OZ_SQ, then for each tile the
+//   digit chunks 0 .. nk-1 for the real part and again for the imaginary part,
+//   which starts with the two chunks still in the buffers;
 //   warp 0 issues the products, part by part, once the accumulators have been
 //   read back;
 //   the last OZ_EW warps read them back (four warps per lane quadrant, 16
-//   columns each): the real part into registers, then the imaginary part, and
-//   with it C += A B^T (OP = +1), C -= A B^T (-1) or C = A B^T (0).
+//   columns each): which entries to sum again, the real part into registers, then
+//   the imaginary part, and with it C += A B^T (OP = +1), C -= A B^T (-1) or C =
+//   A B^T (0).
 //   tile_of(t, I, J)      tile t: A row block I, B row block J
 //   row_of(r, J, cols)    C at the first column of tile column J for row r of
 //                         A (nullptr: no such row), and how
 //                         many of the tile's columns exist
+//   roundings             of C, see oz_below_c
+// The entries that need it are listed, and C left as it was there: oz_redo.
 // smem: OZ_SMEM bytes, 128-byte aligned; the CTA has at least OZ_THREADS
 // threads.  Returns false after a timeout (the caller then calls
 // oz_teardown with failed = true).
 template <int OP, class Tile, class Row>
-__device__ __forceinline__ bool oz_tiles(OzState& st, unsigned char* smem, const unsigned char* imgA,
-                                         const unsigned char* imgB, const int* ea, const int* eb, int nk, long long T,
-                                         long long t_begin, long long t_step, Tile tile_of, Row row_of) {
+__device__ __forceinline__ bool oz_tiles(OzState& st, unsigned char* smem, const OzOperands& im, int K, float roundings,
+                                         long long T, long long t_begin, long long t_step, Tile tile_of, Row row_of) {
   const int tid = threadIdx.x, lane = tid & 31, nwarp = blockDim.x >> 5;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const unsigned s0 = (unsigned)__cvta_generic_to_shared(smem);
@@ -370,22 +517,44 @@ __device__ __forceinline__ bool oz_tiles(OzState& st, unsigned char* smem, const
   // earlier generic-proxy use of this shared memory before the bulk copies write it
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
+  const int nk = (K + OZ_KC - 1) / OZ_KC;
   const long long mine = t_begin < T ? (T - 1 - t_begin) / t_step + 1 : 0;
   const int nl = nk + max(0, nk - 2);  // copies per tile
+  // tiles k0 .. of a group, and those in its buffer q
+  auto group = [&](long long k0) { return (int)min((long long)OZ_SQ, mine - k0); };
+  auto in_buffer = [&](int n, int q) { return min(OZ_SQ / OZ_NBUF, n - q * (OZ_SQ / OZ_NBUF)); };
   if (warp == OZ_LOAD_WARP) {
     if (lane == 0) {
       bool ok = true;
+      int bf = 0;
+      auto next = [&]() {  // the next buffer, free
+        bf = (int)(st.loads % OZ_NBUF);
+        ok = oz_wait(st, OZ_B_FREE + bf);
+        if (!ok) return false;
+        ++st.loads;
+        st.pend |= 1u << (OZ_B_FREE + bf);
+        return true;
+      };
       for (long long k = 0; k < mine && ok; ++k) {
         int I, J;
+        if (k % OZ_SQ == 0) {
+          const int n = group(k);
+          for (int q = 0; q < OZ_NBUF && in_buffer(n, q) > 0 && next(); ++q) {
+            oz_expect(st, bf, in_buffer(n, q) * nk * (OZ_ASUB + OZ_BSUB));
+            for (int t = 0; t < in_buffer(n, q); ++t) {
+              tile_of(t_begin + (k + q * (OZ_SQ / OZ_NBUF) + t) * t_step, I, J);
+              const unsigned dst = s0 + bf * OZ_BUF + t * OZ_SQ_TILE;
+              oz_copy(st, bf, dst, im.sqA + (size_t)I * nk * OZ_ASUB, nk * OZ_ASUB);
+              oz_copy(st, bf, dst + OZ_SQ_A, im.sqB + (size_t)J * nk * OZ_BSUB, nk * OZ_BSUB);
+            }
+          }
+        }
         tile_of(t_begin + k * t_step, I, J);
-        for (int l = 0; l < nl && ok; ++l) {
-          const int c = l < nk ? l : l - nk, bf = (int)(st.loads % OZ_NBUF);
-          ok = oz_wait(st, OZ_B_FREE + bf);
-          if (!ok) break;
-          oz_issue_copy(st, bf, s0 + bf * OZ_BUF, imgA + ((size_t)I * nk + c) * OZ_ACHUNK,
-                        imgB + ((size_t)J * nk + c) * OZ_BCHUNK);
-          ++st.loads;
-          st.pend |= 1u << (OZ_B_FREE + bf);
+        for (int l = 0; l < nl && ok && next(); ++l) {
+          const int c = l < nk ? l : l - nk;
+          oz_expect(st, bf, OZ_BUF);
+          oz_copy(st, bf, s0 + bf * OZ_BUF, im.A + ((size_t)I * nk + c) * OZ_ACHUNK, OZ_ACHUNK);
+          oz_copy(st, bf, s0 + bf * OZ_BUF + OZ_ACHUNK, im.B + ((size_t)J * nk + c) * OZ_BCHUNK, OZ_BCHUNK);
         }
       }
       for (int q = OZ_B_FREE; q < OZ_B_FULL && ok; ++q) ok = oz_wait(st, q);  // the next call starts in step
@@ -393,7 +562,24 @@ __device__ __forceinline__ bool oz_tiles(OzState& st, unsigned char* smem, const
     }
   } else if (warp == OZ_MMA_WARP) {
     bool ok = true;
+    auto full = [&]() {
+      oz_commit(st, OZ_B_FULL);
+      st.pend |= 1u << OZ_B_EMPTY;
+    };
     for (long long k = 0; k < mine && ok; ++k) {
+      if (k % OZ_SQ == 0) {
+        const int n = group(k);
+        ok = __all_sync(0xffffffffu, oz_wait(st, OZ_B_EMPTY));
+        for (int q = 0; q < OZ_NBUF && in_buffer(n, q) > 0 && ok; ++q, ++st.loads) {
+          const int bf = (int)(st.loads % OZ_NBUF);
+          ok = __all_sync(0xffffffffu, oz_wait_phase(st, OZ_B_LOAD + bf));
+          if (!ok) break;
+          for (int t = 0; t < in_buffer(n, q); ++t)
+            oz_issue_squares(st, s0 + bf * OZ_BUF + t * OZ_SQ_TILE, q * (OZ_SQ / OZ_NBUF) + t, nk);
+          oz_commit(st, OZ_B_FREE + bf);
+        }
+        if (ok) full();
+      }
       for (int part = 0; part < 2 && ok; ++part) {
         ok = __all_sync(0xffffffffu, oz_wait(st, OZ_B_EMPTY));
         for (int j = 0; j < nk && ok; ++j) {
@@ -406,10 +592,7 @@ __device__ __forceinline__ bool oz_tiles(OzState& st, unsigned char* smem, const
           oz_issue_mma(st, s0 + bf * OZ_BUF, part, j == 0);
           if (part == 1 || l < nk - 2) oz_commit(st, OZ_B_FREE + bf);  // its last use
         }
-        if (ok) {
-          oz_commit(st, OZ_B_FULL);
-          st.pend |= 1u << OZ_B_EMPTY;
-        }
+        if (ok) full();
       }
       st.loads += nl;
     }
@@ -417,17 +600,61 @@ __device__ __forceinline__ bool oz_tiles(OzState& st, unsigned char* smem, const
     if (!ok) s_fail = 1;
   } else if (warp >= nwarp - OZ_EW) {
     constexpr int CW = OZ_N / (OZ_EW / 4);  // columns per warp
+    static_assert(CW == 16, "oz_ld_squares");
     const int ew = warp - (nwarp - OZ_EW), quad = warp & 3, c0 = CW * (ew >> 2);
     const unsigned acc0 = st.tmem + ((unsigned)(32 * quad) << 16) + (unsigned)c0;
+    auto freed = [&]() {  // the accumulators are in registers
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(st.mb0 + 8 * OZ_B_EMPTY) : "memory");
+    };
+    unsigned long long lossy[2] = {0, 0};  // 16 bits per tile of the group
+    static_assert(OZ_SQ <= 8, "lossy");
     bool ok = true;
     for (long long k = 0; k < mine && ok; ++k) {
       int I, J, cols = 0;
       tile_of(t_begin + k * t_step, I, J);
       const int r = I * OZ_M + 32 * quad + lane;
       c128* crow = row_of(r, J, cols);
-      cols = crow != nullptr ? cols - c0 : 0;
-      const int e_a = cols > 0 ? ea[r] : 0;
-      const int4* ebp = reinterpret_cast<const int4*>(eb + J * OZ_N + c0);
+      cols = crow != nullptr ? max(0, min(CW, cols - c0)) : 0;
+      const int e_a = im.ea[r];
+      const float n_a = im.na[r];
+      const int4* ebp = reinterpret_cast<const int4*>(im.eb + J * OZ_N + c0);
+      const float4* nbp = reinterpret_cast<const float4*>(im.nb + J * OZ_N + c0);
+      // ---- the entries to sum again, of the next OZ_SQ tiles
+      if (k % OZ_SQ == 0) {
+        if (!__all_sync(0xffffffffu, oz_wait_phase(st, OZ_B_FULL))) {
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        lossy[0] = lossy[1] = 0;
+        const int n = group(k);
+#pragma unroll 1
+        for (int t = 0; t < n; ++t) {
+          int It, Jt;
+          tile_of(t_begin + (k + t) * t_step, It, Jt);
+          const float nat = im.na[It * OZ_M + 32 * quad + lane];
+          const float4* nbt = reinterpret_cast<const float4*>(im.nb + Jt * OZ_N + c0);
+          float m2[CW];
+          oz_ld_squares(acc0 + (unsigned)(t * OZ_N), m2);
+          unsigned m = 0;
+#pragma unroll
+          for (int q = 0; q < CW / 4; ++q) {
+            const float4 n4 = nbt[q];
+            const float n_b[4] = {n4.x, n4.y, n4.z, n4.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (oz_lossy(nat, n_b[u], m2[4 * q + u], (float)K)) m |= 1u << (4 * q + u);
+          }
+          if (t < 4) lossy[0] |= (unsigned long long)m << (16 * t);
+          else lossy[1] |= (unsigned long long)m << (16 * (t - 4));
+        }
+        freed();
+      }
+      const int kg = (int)(k % OZ_SQ);
+      unsigned marks = (unsigned)((kg < 4 ? lossy[0] : lossy[1]) >> (16 * (kg & 3))) & ((1u << cols) - 1u);
       double re[CW];
 #pragma unroll 1
       for (int part = 0; part < 2; ++part) {
@@ -448,44 +675,73 @@ __device__ __forceinline__ bool oz_tiles(OzState& st, unsigned char* smem, const
 #pragma unroll
           for (int u = 0; u < 4; ++u) V[4 * q + u] = oz_fixed_sum(d + u, 4);
         }
-        asm volatile("tcgen05.fence::before_thread_sync;");
-        __syncwarp();
-        if (lane == 0)
-          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(st.mb0 + 8 * OZ_B_EMPTY) : "memory");
-        if (cols <= 0) continue;
-        c128* p = crow + c0;
+        freed();
+        if (part == 0) {
 #pragma unroll
-        for (int q = 0; q < CW / 4; ++q, p += 4) {  // four columns; C is read first
-          const int left = cols - 4 * q;
-          if (left <= 0) continue;
-          c128 x[4];
-          if (OP != 0 && part == 1) {
+          for (int q = 0; q < CW / 4; ++q) {
+            const int4 e4 = ebp[q];
+            const int e_b[4] = {e4.x, e4.y, e4.z, e4.w};
 #pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = u < left ? p[u] : mk(0.0, 0.0);
+            for (int u = 0; u < 4; ++u) re[4 * q + u] = oz_to_double(V[4 * q + u], e_a + e_b[u] - 55);
+          }
+          continue;
+        }
+        // C, two columns at a time: an even and an odd lane read and write 32
+        // consecutive bytes of the even lane's row, then of the odd lane's, and
+        // hand each other what belongs to the other's row
+        const bool odd = lane & 1;
+        c128* const other = reinterpret_cast<c128*>(__shfl_xor_sync(0xffffffffu, reinterpret_cast<unsigned long long>(crow), 1));
+        const int ocols = __shfl_xor_sync(0xffffffffu, cols, 1);
+        c128* const pe = (odd ? other : crow) + c0 + (odd ? 1 : 0);  // this lane's column of a pair, in the even row
+        c128* const po = (odd ? crow : other) + c0 + (odd ? 1 : 0);  // and in the odd row
+        const int ce = (odd ? ocols - 1 : cols), co = (odd ? cols - 1 : ocols);  // it exists for columns below
+        auto swap2 = [&](c128 z) {
+          return mk(__shfl_xor_sync(0xffffffffu, z.x, 1), __shfl_xor_sync(0xffffffffu, z.y, 1));
+        };
+#pragma unroll
+        for (int q = 0; q < CW / 4; ++q) {
+          c128 x[4] = {};
+          if (OP != 0) {
+#pragma unroll
+            for (int u = 0; u < 4; u += 2) {
+              const int c = 4 * q + u;
+              c128 ze = mk(0.0, 0.0), zo = ze;
+              if (c < ce) ze = pe[c];
+              if (c < co) zo = po[c];
+              const c128 got = swap2(odd ? ze : zo);
+              x[u] = odd ? got : ze;
+              x[u + 1] = odd ? zo : got;
+            }
           }
           const int4 e4 = ebp[q];
           const int e_b[4] = {e4.x, e4.y, e4.z, e4.w};
-          double v[4];
+          if (OP != 0 && (marks >> (4 * q) & 15u)) {
+            const float4 n4 = nbp[q];
+            const float n_b[4] = {n4.x, n4.y, n4.z, n4.w};
 #pragma unroll
-          for (int u = 0; u < 4; ++u) v[u] = oz_to_double(V[4 * q + u], e_a + e_b[u] - 55);
-          if (part == 0) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) re[4 * q + u] = v[u];
-            continue;
+            for (int u = 0; u < 4; ++u)
+              if (oz_below_c(n_a, n_b[u], roundings, max(oz_exp(x[u].x), oz_exp(x[u].y)), e_a + e_b[u]))
+                marks &= ~(1u << (4 * q + u));
           }
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            if (OP == 0) x[u] = mk(re[4 * q + u], v[u]);
-            else if (OP > 0) x[u] = mk(x[u].x + re[4 * q + u], x[u].y + v[u]);
-            else x[u] = mk(x[u].x - re[4 * q + u], x[u].y - v[u]);
+            const double v = oz_to_double(V[4 * q + u], e_a + e_b[u] - 55);
+            if (marks >> (4 * q + u) & 1u) continue;  // as it was
+            if (OP == 0) x[u] = mk(re[4 * q + u], v);
+            else if (OP > 0) x[u] = mk(x[u].x + re[4 * q + u], x[u].y + v);
+            else x[u] = mk(x[u].x - re[4 * q + u], x[u].y - v);
           }
-          // 16 bytes per access: with a 256-bit store in its place (st.global.v4.f64)
-          // nvcc 13.0.88 left the store out, in code that two kernels of a file call
 #pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (u < left) p[u] = x[u];
+          for (int u = 0; u < 4; u += 2) {
+            const int c = 4 * q + u;
+            const c128 got = swap2(odd ? x[u] : x[u + 1]);
+            if (c < ce) pe[c] = odd ? got : x[u];
+            if (c < co) po[c] = odd ? x[u + 1] : got;
+          }
         }
       }
+      if (!ok) break;
+      if (__any_sync(0xffffffffu, marks != 0)) oz_list_add(im, marks, r, J * OZ_N + c0);
     }
     if (!ok) s_fail = 1;
   }

@@ -121,14 +121,31 @@ __device__ __forceinline__ void latch_status(Control* ctl, int s) {
   atomicCAS(&ctl->status, 0, s);
 }
 
+// Operands of a digit product (ozaki.cuh): digit images, images of the squared magnitudes (one
+// sub-image of 4 or 2 KB per chunk), row exponents, the rows' sums of squared
+// magnitudes, the operands themselves (64 to a row), and the list of entries to sum
+// from these (its length first)
+struct OzOperands {
+  unsigned char* A;
+  unsigned char* B;
+  unsigned char* sqA;
+  unsigned char* sqB;
+  int* ea;
+  int* eb;
+  float* na;
+  float* nb;
+  c128* fa;
+  c128* fb;
+  unsigned* list;
+};
+
 // ---------------------------------------------------------------- context
 struct Layout {
   size_t W, LU, Wlo_re, Wlo_im, X, xa, diag, e, T, v, b, pos_of, scr, part, rec, slots, actg, gsum, gsplit, xs, xadd, cbuf, rbuf,
       snapW, snapState, ctl, total;
   size_t snapW_bytes;  // bytes of the maintained inverse copied by snapshot
   size_t tcimg, tcimgA_bytes, tcimg_bytes;  // mixed path: operand images of the tensor-core fold
-  size_t oz;  // FP64: scratch of the factor (digit images, lists, candidate rows); mixed: without digit images; PEC: digit images
-  size_t ozA, ozB, ozEa, ozEb;  // its digit images and row exponents (the folds of the FP64 search use them too)
+  size_t oz;  // FP64: scratch of the factor (operand images, lists, candidate rows); mixed: without images; PEC: operand images
   size_t X64, last64;  // FP64, PEC: delayed columns (kDelay64 x ldt), index of each pixel's last flip among them
   int ldw, ldl, ldt, R, n_part;
   size_t state_bytes;  // contiguous state block [diag .. b] copied by snapshot
@@ -167,7 +184,9 @@ __host__ __forceinline__ T* at(pngf_ctx* c, size_t off) {
 pngf_status factor_fp64(pngf_ctx* c, const uint8_t* b);
 pngf_status factor_mixed(pngf_ctx* c, const uint8_t* b);
 size_t factor_scratch_bytes(int n, bool images);
-void factor_images(int n, size_t off[5]);  // offsets of the digit images A, B and the row exponents in the scratch, and their end
+// the operand images at the front of that scratch (the folds of the FP64 search use them too), and their bytes
+OzOperands oz_operands(char* scratch, int n);
+size_t oz_operand_bytes(int n);
 // sweep_mixed.cu
 pngf_status run_sweep_mixed(pngf_ctx* c, int n_sweeps, const int32_t* order, int32_t* trace,
                             double* trace_f, int32_t trace_cap, int64_t* counters);

@@ -75,10 +75,7 @@ struct SweepArgs {
   // FP64 path: the delayed set (column i at X64 + i ldt) and the fold's operand images
   c128* X64;
   int* last64;  // n: index of the pixel's last flip in the set, -1: none
-  unsigned char* ozA;
-  unsigned char* ozB;
-  int* ozEa;
-  int* ozEb;
+  OzOperands oz;
   float4* xadd;               // R: alpha_i of the mixed search as double-word pairs, until copied to xa
 };
 
@@ -928,10 +925,7 @@ SweepArgs make_args(pngf_ctx* c) {
   a.xadd = a.mixed ? at<float4>(c, L.xadd) : nullptr;
   a.X64 = at<c128>(c, L.X64);
   a.last64 = at<int>(c, L.last64);
-  a.ozA = reinterpret_cast<unsigned char*>(c->ws + L.ozA);
-  a.ozB = reinterpret_cast<unsigned char*>(c->ws + L.ozB);
-  a.ozEa = at<int>(c, L.ozEa);
-  a.ozEb = at<int>(c, L.ozEb);
+  if (!a.mixed) a.oz = oz_operands(c->ws + L.oz, a.n);
   a.tensor_fold = c->cfg.precision == PNGF_MIXED && c->cfg.tensor_fold;
   a.tcimgA = reinterpret_cast<unsigned char*>(c->ws) + L.tcimg;
   a.tcimgB = a.tcimgA + L.tcimgA_bytes;
