@@ -217,8 +217,8 @@ pngf_status pngf_dbs_sweep(pngf_ctx* ctx, int32_t n_sweeps, const int32_t* order
                            int64_t* counters);
 
 /*
- * Batched DBS: many independent runs advanced by one kernel launch, one CTA
- * per run at a time.  Independent systems exchange nothing: section
+ * Batched DBS: many independent runs advanced by one kernel launch, a CTA or a
+ * small cluster of CTAs per run at a time.  Independent systems exchange nothing: section
  * "Computational efficiency" (and Table 1's footnote on multi-frequency
  * designs) notes that the systems of different frequencies are independent and
  * can be advanced in parallel; here they are independent random starts and/or
@@ -235,12 +235,14 @@ pngf_status pngf_dbs_sweep(pngf_ctx* ctx, int32_t n_sweeps, const int32_t* order
  *   counters  int64 n_ctx x 8 (device, out), per run as in pngf_dbs_sweep
  *   batch_ws  device scratch of pngf_batch_workspace_size(n_ctx) bytes, 256-byte aligned
  * Each run follows the same semantics as pngf_dbs_sweep on its own context.
- * Scheduling (no effect on the results): one CTA per SM takes the runs from a
- * queue in descending n_d (ties in the given order), so that the largest runs
- * start first, each on an SM of its own.
+ * Scheduling: the runs wait in a queue in descending n_d (ties in the given
+ * order), so that the largest runs start first; one CTA per SM, or (FP64, FIRST
+ * mode, few large runs) one cluster of four CTAs on four SMs, takes the next run
+ * whenever it finishes one.  No effect on the results: a run ends bit for bit
+ * alike whatever other runs the call holds.
  */
-/* n_d <= PNGF_BATCH_MAX_ND for every run: the FP64 batch kernel stages one
- * run's gathered column and the column times alpha in 32 x n_d bytes of shared
+/* n_d <= PNGF_BATCH_MAX_ND for every run: in BEST mode the FP64 batch kernel stages
+ * one run's gathered column and the column times alpha in 32 x n_d bytes of shared
  * memory (128 KiB at the bound), so a larger region returns PNGF_EINVAL before
  * any launch. */
 #define PNGF_BATCH_MAX_RUNS 65536

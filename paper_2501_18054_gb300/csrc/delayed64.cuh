@@ -120,6 +120,34 @@ __device__ __forceinline__ c128 delayed_entry(c128 base, const c128* s, int ld) 
   return cadd(base, t[0]);
 }
 
+// ---------------------------------------------------------------- ports
+// o = c_o + G_od (v .* e) over all pixels of a batch's run, by one CTA: the sum's order
+// depends on the CTA's threads only, not on how many CTAs share the run
+__device__ void cta_ports(const SweepArgs& a, const ObjParams& op, c128* s_o, double* s_f) {
+  __shared__ c128 red[kMaxWarps];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int p = 0; p < a.n_o; ++p) {
+    c128 acc = mk(0.0, 0.0);
+    for (int j = threadIdx.x; j < a.n; j += blockDim.x)
+      acc = cfma(a.God[(size_t)p * a.n + j], cmul(a.v[j], a.e[j]), acc);
+    for (int off = 16; off > 0; off >>= 1) {
+      acc.x += __shfl_down_sync(0xffffffffu, acc.x, off);
+      acc.y += __shfl_down_sync(0xffffffffu, acc.y, off);
+    }
+    __syncthreads();
+    if (lane == 0) red[w] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      c128 sum = mk(0.0, 0.0);
+      for (int q = 0; q < nw; ++q) sum = cadd(sum, red[q]);
+      s_o[p] = cadd(a.co[p], sum);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) *s_f = objective_of(op, s_o);
+  __syncthreads();
+}
+
 // ---------------------------------------------------------------- fold
 // Operand images of the fold: A rows y_j = alpha 2^-h x_j, B rows 2^h x_j, where
 // 2^h is about |alpha|^(1/2): both sides then carry the square root of their

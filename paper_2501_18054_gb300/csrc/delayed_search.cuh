@@ -459,12 +459,17 @@ __device__ __forceinline__ bool delayed_search(const SweepArgs& a, const int* fo
       correct_strips<false>(a, pb, pe, a.actg, t_end, reinterpret_cast<float*>(d_smem), OZ_SMEM);
       if (!grid_sync(ctl, P)) { failed = true; break; }
       tick(10);
-      ports_partial(a, pb, pe, cta);
-      if (!grid_sync(ctl, P)) { failed = true; break; }
-      load_state();
-      ports_total(a, s_o, P);
-      if (tid == 0) s_f = objective_of(s_op, s_o);
-      __syncthreads();
+      if (kBatch) {  // every CTA all of it: a run's results do not depend on who shares it
+        load_state();
+        cta_ports(a, s_op, s_o, &s_f);
+      } else {
+        ports_partial(a, pb, pe, cta);
+        if (!grid_sync(ctl, P)) { failed = true; break; }
+        load_state();
+        ports_total(a, s_o, P);
+        if (tid == 0) s_f = objective_of(s_op, s_o);
+        __syncthreads();
+      }
       tick(11);
     }
     if (status == PNGF_ENUMERIC) break;

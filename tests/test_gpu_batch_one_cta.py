@@ -77,3 +77,31 @@ def test_cluster_batch_of_larger_regions(P, sizes):
         for x, z in [(st["diag"], np.diag(Wm)), (st["e"], e), (st["T"], T), (st["W"][iu], Wm[iu]), (c.eval_ports()[0], o)]:
             assert np.max(np.abs(x - z)) <= 1e-12 * np.max(np.abs(z))
         c.close()
+
+
+@pytest.mark.parametrize("sizes,other", [((100, 97, 64), 3), ((300, 120), 3), ((150, 300), 1030)])
+def test_a_run_does_not_depend_on_the_batch_around_it(P, sizes, other):
+    """The same runs on clusters, and on one CTA each (sent there by one more run),
+    with refreshes: the same bits."""
+    def batch(extra):
+        ctxs, orders = [], []
+        for i, n in enumerate(list(sizes) + extra):
+            c = P.DbsContext(_case(n, 3 * n + i, 1 + i % 3), tau=1e-9, refresh_k=5)
+            c.factor(W.random_design(n, i))
+            ctxs.append(c)
+            orders.append(W.shuffled_order(n, 3, seed=i) if i % 2 else None)
+        res = P.DbsBatch(ctxs).dbs_sweep(3, orders=orders)
+        out = [(r["trace"], r["trace_f"], r["counters"], c.state(with_W=True), c.eval_ports(), c.design()) for c, r in zip(ctxs, res)]
+        for c in ctxs:
+            c.close()
+        return out
+
+    for a, b, n in zip(batch([]), batch([other]), sizes):
+        iu = np.triu_indices(n)
+        for x, y in zip(a[:3], b[:3]):
+            assert np.array_equal(x, y)
+        for key in ("diag", "e", "T"):
+            assert np.array_equal(a[3][key], b[3][key])
+        assert np.array_equal(a[3]["W"][iu], b[3]["W"][iu])
+        assert np.array_equal(a[4][0], b[4][0]) and a[4][1] == b[4][1] and np.array_equal(a[5], b[5])
+        assert a[2][4] > 2  # refreshes
