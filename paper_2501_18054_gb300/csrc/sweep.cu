@@ -329,14 +329,7 @@ __global__ void __launch_bounds__(256) accept_prepare_kernel(SweepArgs a, int k,
     c = j >= k ? a.W[(size_t)k * a.ldw + j] : a.W[(size_t)j * a.ldw + k];
     a.cbuf[j] = c;
   }
-  if (threadIdx.x == 0) {
-    const c128 dv = a.dv[k], delta = a.b[k] ? mk(-dv.x, -dv.y) : dv, d = cfms(delta, a.diag[k], mk(1.0, 0.0));
-    const double r = rcp_pos(cabs2(d));
-    s_pv.k = k;
-    s_pv.alpha = cmul(delta, mk(d.x * r, -d.y * r));
-    s_pv.coef = cmul(s_pv.alpha, a.e[k]);
-    FOR_PORTS(p, a.n_o) s_pv.Tk[p] = a.T[(size_t)p * a.ldt + k];
-  }
+  if (threadIdx.x == 0) make_pivot(a, k, s_pv);  // as pngf_score_flips forms it: the scored objective to the bit
   __syncthreads();
   if (ac && j < a.n) ac[j] = cmul(s_pv.alpha, c);
   if (blockIdx.x == 0 && threadIdx.x == blockDim.x - 1) {
