@@ -190,7 +190,8 @@ __device__ bool score_tile_sys(const SweepArgs& a, const ObjParams& op, const c1
 
 // Single-pixel tiles (tile_m = 1), one thread per candidate: the same
 // arithmetic as the warp path for m = 1 (pivot 1 - delta W_kk, its reciprocal,
-// then (delta e_k) times it), so both paths take the same decisions.
+// then (delta e_k) times it, ports of weight zero left out), so both paths take
+// the same decisions.
 __device__ bool score_pixel_tile(const GenArgs& g, const c128 (*s_o)[kMaxPorts], int t, double& F) {
   const int k = g.tiles[t];
   if (k < -1 || k >= g.sys[0].n) {
@@ -204,10 +205,13 @@ __device__ bool score_pixel_tile(const GenArgs& g, const c128 (*s_o)[kMaxPorts],
     const c128 dl = delta_of(a, k);
     const c128 A = csub(mk(1.0, 0.0), cmul(dl, a.diag[k]));
     if (!(cabs2(A) >= 1e-28)) return false;
-    const c128 y = cmul(cmul(dl, a.e[k]), cdiv(mk(1.0, 0.0), A));
+    const c128 y = cmul(cmul(dl, a.e[k]), crecip(A));
     double f = 0.0;
 #pragma unroll 1
-    for (int p = 0; p < a.n_o; ++p) f += objective_term(a.op, p, cadd(s_o[s][p], cmul(a.T[(size_t)p * a.ldt + k], y)));
+    for (int p = 0; p < a.n_o; ++p) {
+      if (a.op.w[p] == 0.0) continue;
+      f += objective_term(a.op, p, cadd(s_o[s][p], cmul(a.T[(size_t)p * a.ldt + k], y)));
+    }
     fs[s] = f;
   }
   F = combine_of(fs, g.n_sys, g.combine, g.kind);
