@@ -350,13 +350,19 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_batch_fp64_kernel(const Swe
     auto fold = [&]() -> bool {
       if (r == 0) return true;
       __syncthreads();
-      fold64_digits(a.X64, ldx, s_al, a.last64, r, n, a.oz, warp, NW);
-      fold64_bases(a.W, a.ldw, a.X64, ldx, s_invd, s_hist, a.last64, nullptr, r, n, tid, blockDim.x);
-      __syncthreads();
-      const bool ok = fold64_product(oz, b_smem, a.W, a.ldw, n, r, a.oz, 0, 1);
-      if (const unsigned m = ok ? oz_listed(a.oz) : 0u) {
-        fold64_redo(a.W, a.ldw, n, r, a.oz, m, warp, NW);
+      bool ok = true;
+      if (fold64_is_direct(r, n)) {
+        fold64_direct(a.W, a.ldw, a.X64, ldx, s_al, s_invd, a.last64, nullptr, r, n, warp, NW);
         __syncthreads();
+      } else {
+        fold64_digits(a.X64, ldx, s_al, a.last64, r, n, a.oz, warp, NW);
+        fold64_bases(a.W, a.ldw, a.X64, ldx, s_invd, s_hist, a.last64, nullptr, r, n, tid, blockDim.x);
+        __syncthreads();
+        ok = fold64_product(oz, b_smem, a.W, a.ldw, n, r, a.oz, 0, 1);
+        if (const unsigned m = ok ? oz_listed(a.oz) : 0u) {
+          fold64_redo(a.W, a.ldw, n, r, a.oz, m, warp, NW);
+          __syncthreads();
+        }
       }
       for (int q = tid; q < n; q += blockDim.x) {
         a.last64[q] = -1;

@@ -197,6 +197,49 @@ __device__ __forceinline__ void fold64_bases(c128* W, int ldw, const c128* X, si
   }
 }
 
+// The fold of a small set, entry by entry in FP64, in place of all of the
+// above: what W(i, j) starts from, then the flips after it.  Warps gw of nw, a row each
+// at a time.  Takes r rank-1 updates on the FP64 pipe: 9 us each at N_d = 1024
+// on 64 CTAs, against some 50 us of a product with its digits and barriers.  Such sets
+// come from kept flips one call at a time and from refreshes every few flips
+// (eight kept flips of a perfect-conductor region in a call each, N_d = 1024: 0.64
+// -> 0.35 ms; 160 runs of 100 pixels refreshed every flip, a CTA each: 35 -> 28 ms, every
+// fourth 13.5 -> 12.2).  The rule holds no grid: a result does not depend on it.
+__device__ __forceinline__ bool fold64_is_direct(int r, int n) { return r <= 2 || (r <= 4 && r * n <= 1024); }
+template <int R>  // an FP64 instruction that a predicate turns off takes its 64 cycles all the same
+__device__ __noinline__ void fold64_direct_of(c128* W, int ldw, const c128* X, size_t ldx, const c128* s_al,
+                                              const c128* inv_d, const int* last, const uint8_t* metal, int n, int gw,
+                                              int nw) {
+  for (int i = gw; i < n; i += nw) {
+    const int li = last[i];
+    c128 y[R];  // alpha x_i
+#pragma unroll
+    for (int q = 0; q < R; ++q) y[q] = cmul(s_al[q], X[(size_t)q * ldx + i]);
+    c128* row = W + (size_t)i * ldw;
+    for (int j = i + (threadIdx.x & 31); j < n; j += 32) {
+      const int lj = last[j], m = max(li, lj);
+      c128 w;
+      if (m < 0) {
+        w = row[j];
+#pragma unroll
+        for (int q = 0; q < R; ++q) w = cfma(y[q], X[(size_t)q * ldx + j], w);
+      } else {
+        w = metal && i == j ? pec_unrotate(inv_d[m], metal[i] != 0) : cmul(X[(size_t)m * ldx + (lj > li ? i : j)], inv_d[m]);
+        for (int q = m + 1; q < R; ++q) w = cfma(cmul(s_al[q], X[(size_t)q * ldx + i]), X[(size_t)q * ldx + j], w);
+      }
+      row[j] = w;
+    }
+  }
+}
+__device__ __forceinline__ void fold64_direct(c128* W, int ldw, const c128* X, size_t ldx, const c128* s_al,
+                                              const c128* inv_d, const int* last, const uint8_t* metal, int r, int n, int gw,
+                                              int nw) {
+  if (r == 1) fold64_direct_of<1>(W, ldw, X, ldx, s_al, inv_d, last, metal, n, gw, nw);
+  else if (r == 2) fold64_direct_of<2>(W, ldw, X, ldx, s_al, inv_d, last, metal, n, gw, nw);
+  else if (r == 3) fold64_direct_of<3>(W, ldw, X, ldx, s_al, inv_d, last, metal, n, gw, nw);
+  else fold64_direct_of<4>(W, ldw, X, ldx, s_al, inv_d, last, metal, n, gw, nw);
+}
+
 // tiles of the upper triangle: row block I (128 rows) against the column
 // blocks J >= 2 I (64 columns)
 __device__ __forceinline__ int fold64_tiles(int n) {

@@ -162,10 +162,25 @@ __device__ __forceinline__ bool delayed_search(const SweepArgs& a, const int* fo
     __syncthreads();
     return true;
   };
+  auto folded = [&]() {  // the set is empty
+    r = 0;
+    for (int jl = tid; jl < own; jl += blockDim.x) {
+      s_last[jl] = -1;
+      a.last64[pb + jl] = -1;
+      s_diag[jl] = a.W[(size_t)(pb + jl) * a.ldw + pb + jl];  // d is formed from the matrix's own diagonal
+    }
+    __syncthreads();
+  };
   // folds the delayed set into W
   auto fold = [&]() -> bool {
     if (r == 0) return true;
     if (!grid_sync(ctl, P)) return false;  // every CTA's part of the columns
+    if (fold64_is_direct(r, n)) {
+      fold64_direct(a.W, a.ldw, a.X64, ldx, s_al, s_invd, a.last64, kPec ? a.b : nullptr, r, n, warp * P + cta, P * NW);
+      if (!grid_sync(ctl, P)) return false;
+      folded();
+      return true;
+    }
     fold64_digits(a.X64, ldx, s_al, a.last64, r, n, a.oz, cta * NW + warp, P * NW);
     fold64_bases(a.W, a.ldw, a.X64, ldx, s_invd, s_hist, a.last64, kPec ? a.b : nullptr, r, n, cta * (int)blockDim.x + tid, P * (int)blockDim.x);
     if (!grid_sync(ctl, P)) return false;
@@ -176,13 +191,7 @@ __device__ __forceinline__ bool delayed_search(const SweepArgs& a, const int* fo
       fold64_redo(a.W, a.ldw, n, r, a.oz, m, warp * P + cta, P * NW);
       if (!grid_sync(ctl, P)) return false;
     }
-    r = 0;
-    for (int jl = tid; jl < own; jl += blockDim.x) {
-      s_last[jl] = -1;
-      a.last64[pb + jl] = -1;
-      s_diag[jl] = a.W[(size_t)(pb + jl) * a.ldw + pb + jl];  // d is formed from the matrix's own diagonal
-    }
-    __syncthreads();
+    folded();
     return true;
   };
   __syncthreads();
@@ -517,7 +526,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_delayed_kernel(const __grid
 
 // CTAs of the delayed search, or 0 where it does not apply (FP64: BEST mode,
 // whose state is checkpointed between single flips, and CTAs asked to hold more
-// pixels than fit; PEC takes more CTAs than asked instead)
+// pixels than fit; PEC takes more CTAs than asked instead).
 int delayed64_grid(pngf_ctx* c) {
   const bool pec = c->cfg.precision == PNGF_PEC;
   if (!pec && c->cfg.mode != PNGF_FIRST_IMPROVEMENT) return 0;
