@@ -526,10 +526,17 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_delayed_kernel(const __grid
 
 // CTAs of the delayed search, or 0 where it does not apply (FP64: BEST mode,
 // whose state is checkpointed between single flips, and CTAs asked to hold more
-// pixels than fit; PEC takes more CTAs than asked instead).
+// pixels than fit; PEC takes more CTAs than asked instead).  Refreshes every few
+// kept flips each fold a small set first and run on fewer CTAs here: the rank-1
+// kernel is the faster one (refresh_k = 1, 2, 4, 8, 16; ms here against there:
+// N_d = 100 3.6, 2.0, 1.7, 1.15, 0.86 against 2.7, 1.8, 1.3, 1.07, 0.96; N_d = 1024
+// 88, 47, 36, 23, 16 against 56, 36, 26, 21, 18; N_d = 4096, from 4: 102, 55, 31
+// against 108, 84, 72).
 int delayed64_grid(pngf_ctx* c) {
   const bool pec = c->cfg.precision == PNGF_PEC;
   if (!pec && c->cfg.mode != PNGF_FIRST_IMPROVEMENT) return 0;
+  const int least_refresh = c->cfg.n_d < 2048 ? 12 : 4;
+  if (!pec && c->cfg.refresh_k > 0 && c->cfg.refresh_k < least_refresh) return 0;
   int g = (c->cfg.n_d + 15) / 16;
   if (g > c->n_sm) g = c->n_sm;
   if (c->cfg.n_ctas > 0 && c->cfg.n_ctas < g) g = c->cfg.n_ctas;
