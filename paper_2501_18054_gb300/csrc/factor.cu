@@ -122,10 +122,13 @@ __device__ void block_inverse(const FactorArgs& a, int m, int bi, int upper, int
 // elimination here is as accurate, but what a search reports there can hang on
 // the last bits of the start state (a metal-filled guide transmits 10^-9 of the
 // power: rounding of 10^-14 in the fields is 10^-9 of it), and stays the same.
+// So does a contrast that is not finite.  (2, from factor_kernel: G is not finite.
+// Eliminating the pixels that are on alone would leave an entry between two
+// others out of sight; the elimination of the whole M meets it and reports it.)
 __global__ void contrast_kernel(const c128* G, const c128* dv, const uint8_t* b, int n, int* high) {
   int h = 0;
   for (int i = threadIdx.x; i < n; i += blockDim.x)
-    if (b[i] && cabs2(dv[i]) * cabs2(G[(size_t)i * n + i]) >= 256.0) h = 1;
+    if (b[i] && !(cabs2(dv[i]) * cabs2(G[(size_t)i * n + i]) < 256.0)) h = 1;
   h = __syncthreads_or(h);
   if (threadIdx.x == 0) *high = h;
 }
@@ -144,7 +147,7 @@ __device__ __forceinline__ bool product_done(const FactorArgs& a, bool ok, int K
 // ---------------------------------------------------------------- the factorisation
 __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_constant__ FactorArgs a) {
   extern __shared__ __align__(128) unsigned char f_smem[];
-  if (*a.high) return;
+  if (*a.high == 1) return;
   __shared__ __align__(8) unsigned long long s_bars[OZ_NBAR];
   __shared__ unsigned s_tmem;
   __shared__ Swaps s_sw;
@@ -159,6 +162,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
   bool ok = true;
   // ---- the lists (CTA 0); one pass over G: Re G + Im G for the refreshes; the rows of W at pixels that are off start as [G | c_d]
   if (cta == 0) factor_lists(a);
+  int bad = 0;
   for (int i = cta; i < n; i += P) {
     const c128* g = a.G + (size_t)i * n;
     c128* w = a.W + (size_t)i * ldw;
@@ -168,6 +172,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
       const c128 z = g[j];
       if (!on) w[j] = z;
       gs[j] = z.x + z.y;
+      bad |= oz_exp(z.x) == 0x7ff || oz_exp(z.y) == 0x7ff;
     }
     if (tid == 0) {
       if (!on) w[n] = a.cd[i];
@@ -177,7 +182,12 @@ __global__ void __launch_bounds__(FT_THREADS, 1) factor_kernel(const __grid_cons
   }
   for (int q = cta * FT_THREADS + tid; q < a.n_o * n; q += P * FT_THREADS)
     a.T[(size_t)(q / n) * a.ldt + q % n] = a.God[q];
+  if (__syncthreads_or(bad) && tid == 0) *const_cast<int*>(a.high) = 2;
   ok = grid_sync(ctl);
+  if (ok && *reinterpret_cast<const volatile int*>(a.high)) {
+    oz_teardown(oz, false);
+    return;
+  }
   const int m = ok ? *reinterpret_cast<volatile int*>(a.count) : 0;
   const int* act = a.act;
   const int* ina = a.act + m;
