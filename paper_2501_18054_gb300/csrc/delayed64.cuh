@@ -70,7 +70,8 @@ template <class TRow>
 __device__ __forceinline__ bool score_pec(const ObjParams& op, bool on, c128 diag, c128 e, TRow T, const c128* o,
                                           double& f_new, c128& alpha, c128& coef, c128& inv_d) {
   const double d2 = cabs2(diag);
-  if (__double_as_longlong(d2) < __double_as_longlong(1e-28)) return false;
+  // a NaN of either sign is no zero pivot: a forced flip reports it as not finite
+  if ((__double_as_longlong(d2) & 0x7fffffffffffffffll) < __double_as_longlong(1e-28)) return false;
   const double r = rcp_pos(d2);
   const c128 sg = mk(diag.x * r, -diag.y * r);
   alpha = mk(-sg.x, -sg.y);

@@ -1,6 +1,6 @@
 """Entries of G that are not finite are reported by the factor wherever they stand, also
 between two pixels that are off (the elimination of the whole system meets them
-as a column without a pivot)."""
+as a column without a pivot), and by the perfect-conductor state when its pivot is."""
 import numpy as np
 import pytest
 
@@ -32,3 +32,15 @@ def test_factor_reports_a_bad_entry_anywhere(P, n, value):
         assert ctx.sync() == P.PNGF_ESINGULAR, (i, j)
         ctx.close()
         case.G_dd[:] = G
+
+
+@pytest.mark.parametrize("value", [np.nan, -np.nan, np.inf])
+def test_perfect_conductor_reports_a_bad_pivot(P, value):
+    case = _case(60, 60, 2)
+    b = W.random_design(60, 1)
+    k = int(np.flatnonzero(b)[3])
+    case.G_dd[k, k] = value
+    ctx = P.DbsContext(case, precision=P.PNGF_PEC)
+    ctx.factor(b)
+    assert ctx.sync() == P.PNGF_ENUMERIC
+    ctx.close()
