@@ -88,7 +88,7 @@ __device__ void block_inverse(const FactorArgs& a, int m, int bi, int upper, int
     auto unit = [&](int r, int cc) { return mk(r == cc ? 1.0 : 0.0, 0.0); };
     c128 l0 = unit(lane, c), l1 = unit(lane, c + 1), h0 = unit(32 + lane, c), h1 = unit(32 + lane, c + 1);
     if (!upper) {
-      for (int k = c; k < BB; ++k) {
+      for (int k = c; k < jb; ++k) {
         const c128 tl = sm[k * (BB + 1) + lane], th = sm[k * (BB + 1) + 32 + lane];
         const c128 s0 = shfl_c(k < 32 ? l0 : h0, k & 31), s1 = shfl_c(k < 32 ? l1 : h1, k & 31);
         if (k < 32) {
@@ -99,7 +99,7 @@ __device__ void block_inverse(const FactorArgs& a, int m, int bi, int upper, int
         h1 = cfms(th, s1, h1);
       }
     } else {
-      for (int k = c + 1; k >= 0; --k) {
+      for (int k = c < jb ? min(c + 1, jb - 1) : -1; k >= 0; --k) {
         const c128 tl = sm[k * (BB + 1) + lane], th = sm[k * (BB + 1) + 32 + lane], d = di[k];
         const c128 s0 = cmul(shfl_c(k < 32 ? l0 : h0, k & 31), d), s1 = cmul(shfl_c(k < 32 ? l1 : h1, k & 31), d);
         if (k >= 32) {
