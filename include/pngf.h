@@ -108,7 +108,8 @@ typedef struct {
                          FP32-pair arithmetic (PNGF_MIXED, a multiple of delay_r) */
   int32_t delay_r;    /* PNGF_MIXED: flips accumulated before the maintained inverse is
                          updated in one rank-delay_r product (1..128); ignored for FP64 */
-  int32_t n_ctas;     /* persistent sweep grid (0 = one per SM, capped by occupancy) */
+  int32_t n_ctas;     /* persistent sweep grid (0 = one per SM, capped by occupancy); FP64 FIRST
+                         and PEC searches take at most n_d / 16 CTAs, PEC at least n_d / 256 */
   double tau;         /* accept iff gain > tau * max(|f|, 1e-30) */
   double obj_weights[PNGF_MAX_PORTS]; /* w_p */
   double s_off[2 * PNGF_MAX_PORTS];   /* c128 per port */
@@ -376,7 +377,7 @@ pngf_status pngf_set_state(pngf_ctx* ctx, const uint8_t* b, const double* W, con
  * Failure-detection controls (the paper has no counterpart).
  *   wait_log2  every bounded device-side wait of this context's later
  *              launches on other CTAs (grid barriers, the word polls of the
- *              mixed search) gives up after 2^wait_log2 polls and latches
+ *              searches; in a batch call, of its run) gives up after 2^wait_log2 polls and latches
  *              PNGF_ETIMEOUT (8..30; 0 = the default 2^24, about ten seconds)
  *   hold_cta   >= 0: CTA hold_cta of the next pngf_dbs_sweep waits, before it
  *              takes part in anything grid-wide, on a flag that nothing sets

@@ -286,10 +286,10 @@ __global__ void __launch_bounds__(kBatchThreads, 2) dbs_batch_kernel(const Sweep
 // barriers, the folds on this SM's tensor core.  The visiting positions are
 // scored kScoreChunk at a time from the current one (a scoring warp on each SM
 // sub-partition; a flip is kept every few positions early in a search).
-// Bound by the SM's FP64 pipe (the columns: r complex multiply-adds per pixel)
-// and the read-back of the folds.  96 lossy-metal runs of 256, 576 and 1024
-// pixels, three sweeps: 734 -> 112 ms (before: the triangle's rank-1 update on
-// the FP64 pipe, 0.6 ms per kept flip of a 1024-pixel run).
+// Bound by the SM's FP64 pipe (the columns: r complex multiply-adds per pixel;
+// the refreshes; the folds' sums in FP64: 81% busy at 1024 lossy-metal pixels) and the
+// read-back of the folds.  76 such runs of ten sweeps take 377 ms, one kept flip 0.25
+// ms (before: the triangle's rank-1 update on the FP64 pipe, 0.6 ms per kept flip).
 constexpr int kScoreChunk = 128;
 
 // the refresh of a whole run by one CTA; smem: the active-pixel list, then the
@@ -521,9 +521,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) dbs_batch_fp64_kernel(const Swe
 // Where the large runs are few: a cluster of kRunCtas CTAs advances one run at a
 // time with the persistent search's own code (delayed_search.cuh; a run's result
 // does not depend on how many CTAs share it).  One CTA per run leaves SMs idle
-// while the large runs last, each bound by the latency of its chain of flips: a
-// 1024-pixel run takes 100 ms on one SM and 50 ms here (96 runs of 256, 576 and
-// 1024 pixels: 109 -> 50 ms).
+// while the large runs last, each bound by its SM's FP64 pipe and the latency of its
+// chain of flips: four 1024-pixel runs of lossy metal take 313 ms on an SM each and
+// 89 ms here, with the FP64 pipes of the four SMs 74% busy.
 constexpr int kRunCtas = 4;
 
 __global__ void __launch_bounds__(OZ_THREADS, 1) __cluster_dims__(kRunCtas, 1, 1)
@@ -582,9 +582,9 @@ size_t batch_workspace_bytes(int n_runs) { return batch_table_bytes(n_runs) + 25
 // largest region's max_n pixels, or 0: one CTA per run.  Measured (ms, clusters
 // against one CTA per run; n_d pixels, 4 / 38 / 76 equal runs of 10 sweeps, refresh
 // every 64 kept flips):
-//   1024: 60 / 109 / 170 against 172 / 198 / 209     100: 0.73 / 2.4 / 3.6 against 1.1 / 3.0 / 3.9
-//    576: 16 / 31 / 49 against 41 / 51 / 52           64: 0.48 / 1.6 / 2.9 against 0.58 / 1.5 / 2.4
-//    256: 2.4 / 6.2 / 10 against 4.6 / 9.3 / 10       16: 0.29 / 1.2 / 2.1 against 0.25 / 1.0 / 1.8
+//   1024: 89 / 157 / 241 against 313 / 370 / 377      100: 0.75 / 2.4 / 3.6 against 1.1 / 3.1 / 4.0
+//    576: 20 / 39 / 64 against 59 / 80 / 82            64: 0.50 / 1.7 / 3.0 against 0.62 / 1.5 / 2.4
+//    256: 2.7 / 6.9 / 11 against 6.4 / 12 / 13         16: 0.29 / 1.2 / 2.2 against 0.27 / 1.0 / 1.7
 // so up to two rounds of clusters over the large runs, and from 96 pixels on.
 // Every CTA holds a share of every run: at least one pixel, at most kOwn64.
 static int batch_clusters(int n_runs, int large, int min_n, int max_n, int n_sm) {

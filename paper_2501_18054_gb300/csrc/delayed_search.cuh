@@ -17,15 +17,16 @@ namespace {
 // pixels lives in shared memory between refreshes.  Grid barriers remain
 // around folds and refreshes.
 //
-// Bound by the latency of that chain, in us per kept flip at N_d = 1024 on 64
-// CTAs: score 1.0, exchange 4.1, fetch 1.4, column 2.5, state 1.0, refresh 1.1,
-// folds 2.1.  Measured against the rank-1 kernel below: N_d = 4096 (dielectric,
-// 10 sweeps) 84.5 -> 17.0 ms, N_d = 1024 (lossy metal) 21.9 -> 12.7 ms, N_d =
-// 100 0.88 -> 0.52 ms.  16 pixels per CTA: a flip's column and state cost the
+// Bound by the latency of that chain, in us per kept flip at N_d = 1024 (lossy
+// metal) on 64 CTAs: score 0.8, exchange 4.3, fetch 1.1, column 2.2, state 0.7,
+// refresh 1.0, folds 3.1 (a fifth of their entries in FP64).  At N_d = 4096 (dielectric,
+// 152 CTAs): 0.9, 4.7, 1.4, 2.6, 0.9, 5.2, 4.0.  Measured against the rank-1 kernel of
+// sweep.cu: N_d = 4096 (10 sweeps) 75.3 -> 18.3 ms, N_d = 1024 23.2 -> 15.7 ms,
+// N_d = 100 0.80 -> 0.53 ms.  16 pixels per CTA: a flip's column and state cost the
 // same for 16 pixels as for one (a warp's FP64 instruction takes 64 cycles
 // whatever its lanes), and fewer CTAs lengthen folds and refreshes more than
-// they shorten the exchange (1024: 12.8 us a flip on 48 CTAs or more, 13.7 on
-// 32, 17.0 on 16).
+// they shorten the exchange (1024, before the folds summed anything in FP64: 12.8 us
+// a flip on 48 CTAs or more, 13.7 on 32, 17.0 on 16).
 constexpr int kOwn64 = 256;  // pixels per CTA, at most
 // word = round sequence number << 32 | key, key = position << 15 | pixel (n_d <= 32768)
 constexpr int kPixBits64 = 15;

@@ -38,7 +38,6 @@ constexpr int BB = 64;        // block of the substitutions, K of their products
 constexpr int FT_THREADS = OZ_THREADS;
 constexpr int FT_WARPS = FT_THREADS / 32;
 
-
 // the ascending lists of the pixels that are on and off (one CTA)
 __device__ void factor_lists(const FactorArgs& a) {
   __shared__ int s_scan[FT_WARPS];

@@ -22,8 +22,8 @@
 //
 // The initial state of a design is built from the empty design (S = G, u =
 // c_d, v = G_od) by adding its metal pixels one by one (forced flips).
-// N_d = 1024, start built and three sweeps: 51.1 ms with H, Q and W updated one
-// flip at a time, 12.0 ms now (about 12 us a flip, the chain of the search).
+// N_d = 1024, start built and three sweeps: 54.1 ms with H, Q and W updated one
+// flip at a time, 15.1 ms now (the chain of the search for each flip).
 #include <cstdio>
 
 #include "delayed_search.cuh"

@@ -1,6 +1,7 @@
 // Direct binary search on the device (FP64 path).  FIRST mode runs on the
 // delayed-update kernel of delayed_search.cuh; the rank-1 kernel below serves BEST
-// mode and contexts whose CTAs hold more pixels than that kernel takes.  Both
+// mode, refreshes every few kept flips, and contexts whose CTAs hold more pixels
+// than that kernel takes (delayed64_grid).  Both
 // follow the same steps; single kept flips (pngf_accept_flip) are at the end.
 //
 // Per kept flip of pixel k (section "Low-rank update evaluation", Eqs. 9-14 in
@@ -19,8 +20,8 @@
 //
 // One cooperative launch runs the whole search.  In the rank-1 kernel pixels are split into
 // contiguous chunks, one per CTA; the packed upper triangle of W is split
-// into equal element ranges, one per CTA.  Grid-wide barriers are a counter
-// plus generation word with a bounded spin: a barrier that waits longer than
+// into equal element ranges, one per CTA.  Grid-wide barriers are one arrival
+// counter with a bounded spin: a barrier that waits longer than
 // the spin limit latches PNGF_ETIMEOUT and every CTA returns.
 #include <cstdio>
 #include <mutex>
@@ -345,7 +346,7 @@ __global__ void __launch_bounds__(256) accept_prepare_kernel(SweepArgs a, int k,
 // A warp takes 128 columns of one row at a time: four independent 512-byte
 // reads in flight, and alpha c_i once per row piece (from `ac`, or formed here
 // where the caller has no room for it).  Bound by the FP64 pipe, one complex
-// FMA per element: 14 us at N_d = 2112, where a flip takes 32 us with its two
+// FMA per element: 14 us at N_d = 2112, where a flip takes 33 us with its two
 // launches (about 52 with alpha c_i formed per element, in three launches).
 // 256 columns a piece: 36 us (half the CTAs fit an SM).
 constexpr int kPiece = 128;
