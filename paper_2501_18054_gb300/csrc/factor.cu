@@ -117,10 +117,14 @@ __device__ void block_inverse(const FactorArgs& a, int m, int bi, int upper, int
 }
 
 // Whether a pixel that is on has |dv G_kk| >= 16: lossy metal (500) and the
-// like, against 0.5 for eps = 10.  Such systems go to factor_pipe.cu.  The
-// elimination here is as accurate, but what a search reports there can hang on
-// the last bits of the start state (a metal-filled guide transmits 10^-9 of the
-// power: rounding of 10^-14 in the fields is 10^-9 of it), and stays the same.
+// like, against 0.5 for eps = 10.  Such systems go to factor_pipe.cu.  Not for
+// accuracy: at N_d = 576 and contrasts of 0.5 to 500 (both devices, dv scaled, four
+// designs) the error of W here is 3e-16 to 6e-16 against 7e-16 to 1e-15 there (the guide at
+// 0.5: 4e-15 each; at 2, near a resonance: 2e-13 against 3e-13), that of the objective
+// within a factor of four either way, and the time 3.2-3.6 ms against 13.3.  But
+// what a search reports on metal can hang on the last bits of the start state (a
+// metal-filled guide transmits 10^-9 of the power: rounding of 10^-14 in the fields is
+// 10^-9 of it), and stays the same; any line between the two contrasts does that.
 // So does a contrast that is not finite.  (2, from factor_kernel: G is not finite.
 // Eliminating the pixels that are on alone would leave an entry between two
 // others out of sight; the elimination of the whole M meets it and reports it.)
